@@ -394,7 +394,16 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
   // dense_ids: polynomial products on the dense path (output-block tasks);
   // hash_ids: everything accumulated by tiles of term pairs (hash products and
   // Poisson products on the dense path); hll_ids: products with a hash table
-  std::vector<int> live_ids, dense_ids, hash_ids, hll_ids;
+  // win_ids: products accumulated by key windows (neither list's arrays)
+  std::vector<int> live_ids, dense_ids, hash_ids, hll_ids, win_ids[2];
+  double win_bound = 0.0;
+  for (int p = 0; p < nprod; ++p) {
+    if (ctx->split_hist) plans[p].p.win.kind = 0;   // samples the operands only
+    if (plans[p].st == KR_OK && !plans[p].empty && plans[p].p.win.kind)
+      win_bound += 32.0 * std::min((plans[p].p.nt > 0 ? 2.0 : 1.0) * (double)plans[p].p.f.n * (double)plans[p].p.g.n,
+                                   (double)plans[p].p.kspan);
+  }
+  const bool win_estimate = win_bound > WIN_BOUND_BYTES;
   for (int p = 0; p < nprod; ++p) {
     if (plans[p].st != KR_OK) continue;
     if (plans[p].empty) {   // truncated to nothing: a zero product
@@ -403,10 +412,18 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       continue;
     }
     live_ids.push_back(p);
+    if (plans[p].p.win.kind) {
+      win_ids[plans[p].p.win.kind - 1].push_back(p);
+      if (win_estimate) hll_ids.push_back(p);
+      continue;
+    }
     const bool block = plans[p].p.path == PATH_DENSE && plans[p].p.nt == 0;
     (block ? dense_ids : hash_ids).push_back(p);
     if (plans[p].p.path == PATH_HASH) hll_ids.push_back(p);
   }
+  // the windows' terms follow the compacted ones in the output arrays
+  std::stable_sort(live_ids.begin(), live_ids.end(),
+                   [&](int a, int b) { return plans[a].p.win.kind < plans[b].p.win.kind; });
   const int nlive = (int)live_ids.size();
   if (nlive == 0) return;
   std::vector<int> local(nprod, -1);
@@ -416,6 +433,27 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
   for (int p : hash_ids) h_hash_local.push_back(local[p]);
   std::vector<int32_t> h_hll_local;
   for (int p : hll_ids) h_hll_local.push_back(local[p]);
+  std::vector<int32_t> h_win_local;
+  int64_t win_cap_total = 0, win_cap_total1 = 0, win_max_terms = 0, win_max_samples = 0, win_max_bins = 0;
+  bool win_poisson = false;
+  std::vector<int> win_merge[2];   // merging products, by position in their kind's list
+  int win_stage = 0;
+  for (const auto& ids : win_ids)
+    for (int p : ids) {
+      const Prod& P = plans[p].p;
+      h_win_local.push_back(local[p]);
+      win_cap_total += P.win.cap;
+      if (P.win.kind == WIN_32) win_cap_total1 += P.win.cap;
+      win_max_terms = std::max(win_max_terms, std::max(P.f.n, P.g.n));
+      win_max_samples = std::max(win_max_samples, P.win.samples);
+      win_max_bins = std::max(win_max_bins, P.win.nbins);
+      win_poisson |= P.nt > 0;
+      if (P.win.merge) {
+        const int k = P.win.kind - 1;
+        win_merge[k].push_back((int)h_win_local.size() - 1 - (k ? (int)win_ids[0].size() : 0));
+      }
+      win_stage = std::max(win_stage, (int)P.win.stage);
+    }
   // deferred: one product, no hash table (nothing to size from the estimate or
   // to regrow), not a prepared or split run.  Its whole plan (phases B1 and
   // B2) goes to the device in one copy, and no step waits for the device
@@ -435,6 +473,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     Prod* lprods; OpRef* oplists; int32_t* dense_ids; int64_t* block_begin; int32_t* hash_ids;
     int64_t* task_begin; int64_t* scan; DenseTask* tasks; uint32_t* hll; size_t hll_bytes;
     int32_t* hll_ids; int64_t* hll_task_begin; int64_t* chunk_begin; unsigned long long* split; char* up_end;
+    int32_t* win_ids; int64_t* win_prefix[2]; char* win_zero; size_t win_zero_bytes; unsigned int* win_done;
   } A{};
   for (int pass = 0; pass < 2; ++pass) {
     Bump b(pass ? ctx->work : nullptr);
@@ -448,11 +487,41 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     A.hll_ids = b.take<int32_t>((int64_t)hll_ids.size() + 1);
     A.hll_task_begin = b.take<int64_t>((int64_t)hll_ids.size() + 1);
     A.chunk_begin = b.take<int64_t>((int64_t)nlive + 1);   // used by a deferred product
+    A.win_ids = b.take<int32_t>((int64_t)h_win_local.size() + 1);
     A.up_end = b.base ? b.base + b.off : nullptr;
     A.scan = b.take<int64_t>(scan_b1 + 1);
     A.tasks = b.take<DenseTask>(dense_tasks_total);
     A.hll = b.take<uint32_t>((int64_t)hll_ids.size() * HLL_M);
     A.hll_bytes = sizeof(uint32_t) * hll_ids.size() * HLL_M;
+    // windowed products: what the planning kernels need cleared, contiguous
+    b.off = (b.off + 255) / 256 * 256;
+    A.win_zero = b.base ? b.base + b.off : nullptr;
+    {
+      const size_t zero_start = b.off;
+      A.win_done = b.take<unsigned int>(2);
+      for (const auto& ids : win_ids)
+        for (int p : ids) {
+          plans[p].p.win.desc = b.take<WinDesc>(1);
+          plans[p].p.win.hist = b.take<uint32_t>(plans[p].p.win.nbins);
+        }
+      A.win_zero_bytes = h_win_local.empty() ? 0 : b.off - zero_start;
+    }
+    for (int k = 0; k < 2; ++k) A.win_prefix[k] = b.take<int64_t>((int64_t)win_ids[k].size() + 1);
+    for (const auto& ids : win_ids)
+      for (int p : ids) {
+        Prod& P = plans[p].p;
+        P.win.start = b.take<int64_t>(P.win.cap + 1);
+        P.win.run = b.take<int32_t>(P.win.cap + 1);
+        P.win.before = b.take<uint32_t>(P.win.cap + 1);
+        P.win.idx = b.take<int32_t>(2 * (P.win.idx_cap + 2));
+        if (P.nt > 0) {
+          const int64_t na = P.win.swap ? P.g.n : P.f.n, nb = P.win.swap ? P.f.n : P.g.n;
+          P.win.acode = b.take<int64_t>(2 * na);
+          P.win.acoef = b.take<double>(na);
+          P.win.bcode = b.take<int64_t>(2 * nb);
+          P.win.bcoef = b.take<double>(2 * nb);
+        }
+      }
     A.split = ctx->split_hist ? b.take<unsigned long long>(ctx->split_nbins) : nullptr;
     for (int q = 0; q < (int)hll_ids.size(); ++q)
       if (pass) plans[hll_ids[q]].p.hll = A.hll + (int64_t)q * HLL_M;
@@ -508,6 +577,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
   struct B2 {
     int64_t* chunk_begin; int64_t* counts; int64_t* scan; int64_t* bins; uint64_t *okey, *oval, *okey2, *oval2;
     int64_t* counters; uint64_t* cstat; char* zero; size_t zero_bytes;
+    int64_t* wtotal; unsigned char* wstage; WinOut wout[2]; int64_t *wbefore, *wscan;
   } Z{};
   int64_t out_total = 0, nchunks_total = 0, bins_total = 0, scan_b2 = 0, max_hash_out = 0;
   std::vector<int64_t> h_chunk_begin(nlive + 1, 0);
@@ -516,6 +586,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     for (int p : hll_ids) {
       Plan& pl = plans[p];
       finish_hash_sizes(ins[p].opts, &pl);
+      if (pl.p.win.kind) continue;   // its terms come out ordered
       max_hash_out = std::max(max_hash_out, pl.out_cap);
       const int64_t nb = order_bins(pl.p.kspan);
       if (order_buckets(pl.p.kspan) <= ORDER_MAX_BUCKETS)
@@ -542,6 +613,22 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       Z.chunk_begin = b.take<int64_t>(nlive + 1);
       Z.counts = b.take<int64_t>(nchunks_total + 1);
       Z.scan = b.take<int64_t>(std::max(scan_b2, scan_scratch_entries(nchunks_total)) + 1);
+      // windowed products: raw terms, stretches and scan scratch
+      Z.wtotal = b.take<int64_t>(2);
+      Z.wbefore = b.take<int64_t>(std::max(win_cap_total1, win_cap_total - win_cap_total1));
+      Z.wscan = b.take<int64_t>(h_win_local.empty() ? 0 : scan_scratch_entries(win_cap_total));
+      for (int k = 0; k < 2; ++k) {
+        WinOut& O = Z.wout[k];
+        const int64_t nw = k ? win_cap_total - win_cap_total1 : win_cap_total1;
+        int64_t terms = 0;
+        for (int p : win_ids[k]) terms += plans[p].out_cap;
+        O.cap = terms;
+        O.key = b.take<uint64_t>(terms);
+        O.val = b.take<uint64_t>(terms);
+        O.nseg = nw ? 16 * nw + 4096 : 0;
+        O.seg = b.take<WinSeg>(O.nseg);
+      }
+      Z.wstage = b.take<unsigned char>((int64_t)win_staging(win_stage, ctx->num_sms));
       Z.bins = b.take<int64_t>(bins_total);
       Z.okey = b.take<uint64_t>(out_total);
       Z.oval = b.take<uint64_t>(out_total);
@@ -551,10 +638,18 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       b.off = (b.off + 255) / 256 * 256;
       const size_t zero_start = b.off;
       Z.zero = b.base ? b.base + zero_start : nullptr;
-      Z.counters = b.take<int64_t>(4);   // dense task queue (2), compaction ticket and error flag
+      Z.counters = b.take<int64_t>(6);   // dense task queue (2), compaction ticket and error flag, window tickets
+      for (int k = 0; k < 2; ++k) {
+        WinOut& O = Z.wout[k];
+        const int64_t nw = k ? win_cap_total - win_cap_total1 : win_cap_total1;
+        O.used = b.take<unsigned long long>(2);
+        O.count = b.take<int64_t>(nw);
+        O.head = b.take<int32_t>(nw);
+      }
       Z.cstat = b.take<uint64_t>(nchunks_total + 1);
       for (int p : live_ids) {
         Plan& pl = plans[p];
+        if (pl.p.win.kind) continue;
         if (pl.p.path == PATH_DENSE && pl.p.nt > 0) pl.p.dense = (void*)b.take<uint64_t>(pl.p.kspan);
         else if (pl.p.path != PATH_DENSE) pl.p.table = b.take<uint64_t>(2 * pl.p.slots);
       }
@@ -641,6 +736,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     put(A.hll_ids, h_hll_local.data(), 4 * h_hll_local.size());
     put(A.hll_task_begin, h_hll_task_begin.data(), 8 * h_hll_task_begin.size());
     put(A.chunk_begin, h_chunk_begin.data(), 8 * h_chunk_begin.size());
+    put(A.win_ids, h_win_local.data(), 4 * h_win_local.size());
     ck(ctx, cudaMemcpyAsync(dbase, st, span, cudaMemcpyHostToDevice, s), "upload plan");
   }
   const OpRef* d_all = A.oplists;
@@ -741,6 +837,18 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       mark(ctx, s, "hll");
     }
   }
+  if (!h_win_local.empty()) {
+    ck(ctx, cudaMemsetAsync(A.win_zero, 0, A.win_zero_bytes, s), "memset window plan");
+    for (int k = 0, at = 0; k < 2; at += (int)win_ids[k].size(), ++k) {
+      if (win_ids[k].empty()) continue;
+      ck(ctx, launch_win_plan(A.lprods, A.win_ids + at, (int)win_ids[k].size(), win_poisson,
+                              win_merge[k].data(), (int)win_merge[k].size(), win_max_terms, win_max_samples, win_max_bins, A.win_prefix[k], k ? WIN_SLOTS_64 : WIN_SLOTS_32,
+                              (int64_t)ctx->num_sms * WIN_CTAS_PER_SM, A.win_done + k, s),
+         "window plan");
+      ctx->launches += 3 + (win_poisson ? 1 : 0) + (win_merge[k].empty() ? 0 : 1 + (int)win_merge[k].size());
+    }
+    mark(ctx, s, "window_plan");
+  }
   if (!ctx->replay && !deferred) {
     ck(ctx, cudaMemcpyAsync(hl, A.lprods, sizeof(Prod) * nlive, cudaMemcpyDeviceToHost, s), "download");
     ck(ctx, cudaStreamSynchronize(s), "sync b1");
@@ -826,11 +934,25 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       }
     }
     int compact_launches = 0;
-    ck(ctx, launch_compact(A.lprods, nlive, Z.chunk_begin, nchunks_total, Z.counts, Z.cstat, Z.counters + 2,
+    const bool compacted = (int)h_win_local.size() < nlive;
+    if (compacted) ck(ctx, launch_compact(A.lprods, nlive, Z.chunk_begin, nchunks_total, Z.counts, Z.cstat, Z.counters + 2,
                            Z.scan, Z.okey, Z.oval, out_total, s, direct, &compact_launches),
        "compaction");
     ctx->launches += compact_launches;
-    mark(ctx, s, "compact");
+    if (compacted) mark(ctx, s, "compact");
+    const int64_t* wbase = compacted ? Z.counts + nchunks_total : nullptr;
+    for (int k = 0, at = 0; k < 2; at += (int)win_ids[k].size(), ++k) {
+      if (win_ids[k].empty()) continue;
+      int wl = 0;
+      ck(ctx, launch_window(A.lprods, A.win_ids + at, A.win_prefix[k], (int)win_ids[k].size(), k + 1,
+                            k ? win_cap_total - win_cap_total1 : win_cap_total1, Z.counters + 4 + k, Z.wout[k],
+                            Z.wbefore, Z.wscan, wbase, Z.wtotal + k, out_total, Z.okey, Z.oval, Z.wstage,
+                            win_stage, ctx->num_sms, s, &wl),
+         "window accumulate");
+      wbase = Z.wtotal + k;
+      ctx->launches += wl;
+      mark(ctx, s, "hash_insert");
+    }
     if (deferred) {
       // the count, the status and the position (0: the only product) stay on
       // the device; the decode reads them there
@@ -866,7 +988,8 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       Prod& P = hl2[q];
       plans[p].p.nout = P.nout;
       plans[p].p.out_start = P.out_start;
-      if (!ctx->replay && (P.status & ST_OUTCAP) && !(P.status & ~ST_OUTCAP) && !plans[p].outcap_full) {
+      if (!ctx->replay && !plans[p].outcap_full && !(P.status & ~ST_OUTCAP) &&
+          ((P.status & ST_OUTCAP) || (P.win.kind && P.nout > P.out_cap))) {
         // the estimate fell short: rerun with room for a full table
         plans[p].outcap_full = true;
         plans[p].p.status = 0;
@@ -899,7 +1022,9 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     for (int q = 0; q < nlive; ++q) {
       const int p = live_ids[q];
       ProdResult& r = res[p];
-      if (r.st != KR_OK || r.prod.path != PATH_HASH || r.n < 2 || ins[p].opts.unsorted) continue;
+      if (r.st != KR_OK || r.prod.path != PATH_HASH || r.prod.win.kind || r.n < 2 ||
+          ins[p].opts.unsorted)
+        continue;
       uint64_t* k = Z.okey + r.prod.out_start;
       uint64_t* v = Z.oval + r.prod.out_start;
       uint64_t* k2 = Z.okey2;

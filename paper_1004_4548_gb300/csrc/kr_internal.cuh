@@ -95,6 +95,72 @@ struct Operand {
   unsigned char* mtmp;
 };
 
+// Windowed accumulation (kr_window.cu): a list of ascending codes searched by
+// key window, with its bucket index (idx[b] = first entry >= b << shift).
+struct WinList {
+  const int64_t* code;   // relative to base
+  const void* coef;
+  const int32_t* idx;
+  int64_t n, nidx, base, span;   // span: the last code
+  int64_t nv;            // Poisson: the first nv entries stand for difference terms
+  int32_t shift;
+};
+
+// Written on the device by the window planning.
+struct WinDesc {
+  WinList L[2];          // the polynomial's list, or the cosines' and the sines'
+  int64_t na, nca;       // terms of the walked factor, and its cosines
+  int64_t nw;            // windows
+  float total;           // samples of the histogram
+  float rs[16], rn[16];  // by region of the windows: sum of 1 / (pairs sharing a sampled pair's key), samples
+};
+constexpr int WIN_REGIONS = 16;
+constexpr int WIN_CTAS_PER_SM = 2;
+constexpr int WIN_STAGE_MAX = 32;
+
+// windowed accumulation of a product: offsets within a window of 32 or 64 bits
+constexpr int WIN_32 = 1, WIN_64 = 2;
+constexpr int WIN_SLOTS_32 = 8192, WIN_SLOTS_64 = 4096;   // table slots (96 KB, 64 KB)
+
+// Raw output of the windows: terms in stretches, and per run (by its first
+// window) the list of its stretches in key order.
+struct WinSeg {
+  int64_t pos;
+  int32_t n, next;       // next: index of the run's next stretch, -1 at its end
+};
+struct WinOut {
+  uint64_t* key;         // [cap]
+  uint64_t* val;
+  int64_t cap;
+  WinSeg* seg;           // [nseg]
+  int64_t nseg;
+  int32_t* head;         // per window, zeroed: index + 1 of its run's first stretch
+  int64_t* count;        // per window, zeroed: terms of its run
+  unsigned long long* used;   // [2], zeroed: terms, stretches
+};
+
+// A windowed product's plan (host) and scratch.
+struct Win {
+  int32_t kind;          // 0: not windowed
+  int32_t swap;          // 1: g is walked and f searched (the shorter factor is walked)
+  int32_t merge;         // a CTA may take several windows at once
+  int32_t sparse;        // (not merging) most pairs have a key of their own
+  int32_t stage;         // windows of a staged run (0: none)
+  int32_t bin_shift;     // histogram bins of 2^bin_shift keys
+  int64_t nbins, nw, samples, cap, idx_cap, pt;   // pt: pairs per window
+  uint32_t* hist;        // [nbins], zeroed
+  float updates;         // pairs (Poisson: both terms of each)
+  int64_t* start;        // [cap + 1] first keys of the windows
+  uint32_t* before;      // [cap + 1] histogram samples before each
+  int32_t* run;          // [cap + 1] first windows of the runs
+  WinDesc* desc;
+  int32_t* idx;          // [2][idx_cap + 2]
+  int64_t* acode;        // Poisson: [2][na] codes and mirrored codes of the walked factor
+  double* acoef;         // Poisson: [na] its coefficients in the mirrored order
+  int64_t* bcode;        // Poisson: [2 nb] codes of both searched lists
+  double* bcoef;         // Poisson: [2 nb]
+};
+
 // One product, planned on the host, read by every kernel.
 struct Prod {
   Operand f, g;
@@ -156,6 +222,7 @@ struct Prod {
   int64_t tiles_j;      // tiles along g
   int64_t task_begin;   // first task index of this product (hash tiles)
   int64_t ntasks;
+  Win win;
   // compaction
   int64_t chunk;        // accumulator slots per compaction chunk
   int64_t nchunks;
@@ -434,6 +501,22 @@ cudaError_t launch_probe_table_update(uint64_t* table, uint64_t slots, int64_t d
 // kernel of their own)
 cudaError_t launch_hash_insert(Prod* dprods, const int32_t* dhash_prods, const int64_t* dtask_begin,
                                int nhash, bool poly, bool pseries, bool trunc, int grid, cudaStream_t s);
+// Windowed accumulation: lists, bucket indexes, histogram and cuts of every
+// listed product (drprefix: nwp + 1 offsets of runs; ddone: a zeroed counter;
+// merging: positions in the list of the `merge` products with Win::merge),
+// then the windows of the products of one kind (max_windows: at most that many)
+// and the copy that puts the products together.  dbefore, dscan: max_windows
+// int64 and a scan's scratch; dbase: where the terms start (null: 0); *dtotal:
+// where they end.
+cudaError_t launch_win_plan(const Prod* dprods, const int32_t* dwprods, int nwp, bool poisson,
+                            const int* merging, int merge,
+                            int64_t max_terms, int64_t max_samples, int64_t max_bins, int64_t* drprefix,
+                            int64_t slots, int64_t ctas, unsigned int* ddone, cudaStream_t s);
+cudaError_t launch_window(Prod* dprods, const int32_t* dwprods, const int64_t* drprefix, int nwp, int kind,
+                          int64_t max_windows, int64_t* dticket, const WinOut& out, int64_t* dbefore, int64_t* dscan,
+                          const int64_t* dbase, int64_t* dtotal, int64_t cap, uint64_t* okey, uint64_t* oval,
+                          unsigned char* staging, int stage_max, int sms, cudaStream_t s, int* launches);
+size_t win_staging(int stage_max, int sms);   // bytes of launch_window's staging for the largest Win::stage
 // Compaction: up to this many chunks one pass (each chunk read once, one
 // launch); above it two passes, whose counting pass keeps more loads in
 // flight.

@@ -57,6 +57,53 @@ static void plan_sort(Operand& op, int64_t key_range, int* passes, int64_t* radi
   }
 }
 
+// Windowed accumulation (kr_window.cu), where it applies: hash products, and
+// Poisson products whose key array would be sparsely hit, unless the caller
+// sized a table or the product is truncated by a criterion that the windows
+// cannot apply by key alone.
+static void plan_window(const kr_opts& o, Plan* out) {
+  Prod& P = out->p;
+  P.win = Win{};
+  if (P.ctrunc || P.htrunc || (P.graded && P.nt > 0)) return;
+  if (o.table_slots > 0 || o.probe_limit > 0 || o.max_regrow != 0) return;
+  const double m = P.nt > 0 ? 2.0 : 1.0;
+  const double updates = m * (double)P.f.n * (double)P.g.n;
+  if (P.path == PATH_DENSE && (double)P.kspan < 0.5 * updates) return;
+  const int64_t na = std::min(P.f.n, P.g.n), nb = std::max(P.f.n, P.g.n);
+  if (nb > WIN_MAX_LIST || m * (double)na > WIN_MAX_WALK) return;
+  Win& W = P.win;
+  W.swap = P.g.n < P.f.n ? 1 : 0;
+  // pairs per window: as many as keep the table about half full where every
+  // pair has a key of its own, fewer where the product has few windows
+  const double fill = 0.49;
+  double pt = fill * WIN_SLOTS_32;
+  W.kind = (double)P.kspan / std::max(1.0, updates / pt) < 67108864.0 ? WIN_32 : WIN_64;
+  if (W.kind == WIN_64) pt = fill * WIN_SLOTS_64;
+  const int64_t slots = W.kind == WIN_64 ? WIN_SLOTS_64 : WIN_SLOTS_32;
+  W.merge = updates > 600.0 * pt;
+  // staged runs: many windows, each with fewer than two pairs per term walked;
+  // as many windows a run as make up four times as many pairs as terms walked,
+  // at least 8 (8 keep the staging of all CTAs near the size of L2)
+  const double walk = m * (double)na;
+  if (updates > 8.0 * 600.0 * pt && pt < 2.0 * walk)
+    W.stage = (int32_t)std::min((double)WIN_STAGE_MAX, std::max(8.0, std::ceil(4.0 * walk / pt)));
+  W.updates = (float)updates;
+  W.pt = (int64_t)pt;
+  W.nw = std::max<int64_t>(1, (int64_t)(updates / pt));
+  W.samples = (int64_t)std::min((double)P.f.n * (double)P.g.n, std::min(16777216.0, std::max(4096.0, 96.0 * (double)W.nw)));
+  int sh = 0;
+  while ((int64_t(1) << sh) < slots) ++sh;   // no window below the directly addressed size
+  while (((P.kspan - 1) >> sh) + 1 > std::min<int64_t>(WIN_MAX_BINS, 8 * W.nw)) ++sh;
+  W.bin_shift = sh;
+  W.nbins = ((P.kspan - 1) >> sh) + 1;
+  W.cap = 3 * W.nw + 16;
+  W.idx_cap = std::min<int64_t>(65536, std::max<int64_t>(64, next_pow2(2 * nb)));
+  P.slots = 0;
+  P.nchunks = 0;
+  out->out_cap = (int64_t)std::min(updates, (double)P.kspan);
+  out->accum_bytes = 0;
+}
+
 void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_sms, Plan* out) {
   Plan& pl = *out;
   pl = Plan();
@@ -263,6 +310,7 @@ void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_
     P.chunk = COMPACT_CHUNK;
     P.nchunks = ceil_div(P.kspan, P.chunk);
     pl.out_cap = (int64_t)std::min((double)P.kspan, 2.0 * pairs);
+    plan_window(o, &pl);
   } else if (P.path == PATH_DENSE) {
     int64_t S = o.block_slots > 0 ? o.block_slots : DEFAULT_S;
     if (S < 256) S = 256;
@@ -304,11 +352,17 @@ void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_
     P.ntasks = ceil_div(nf, HASH_TILE_I) * P.tiles_j;
     P.chunk = COMPACT_CHUNK_HASH;
     // table size, chunks and output capacity follow in finish_hash_sizes
+    plan_window(o, &pl);
   }
 }
 
 void finish_hash_sizes(const kr_opts& o, Plan* pl) {
   Prod& P = pl->p;
+  if (P.win.kind) {   // no table; the estimate, where there is one, bounds the output room
+    const double all = std::min((P.nt > 0 ? 2.0 : 1.0) * (double)P.f.n * (double)P.g.n, (double)P.kspan);
+    pl->out_cap = (int64_t)(P.hll_est > 0.0 && !pl->outcap_full ? std::min(all, P.hll_est * 1.1 + 4096.0) : all);
+    return;
+  }
   const double m = P.nt > 0 ? 2.0 : 1.0;
   const double upper = std::min(m * (double)P.f.n * (double)P.g.n, (double)P.kspan);
   const double alpha = o.load_factor > 0.0 && o.load_factor <= 0.9 ? o.load_factor : DEFAULT_LOAD;

@@ -31,6 +31,15 @@ constexpr int64_t COMPACT_CHUNK = 8192;
 constexpr int64_t COMPACT_CHUNK_HASH = 4096;
 constexpr double DEFAULT_LOAD = 0.5;
 constexpr int DEFAULT_PROBES = 512;
+// windowed accumulation: terms of the searched factor, and of the walked one
+// (walked once per window, so its length against a window's pairs bounds the
+// searches that find nothing)
+constexpr int64_t WIN_MAX_LIST = int64_t(1) << 20;
+constexpr double WIN_MAX_WALK = 65536.0;
+constexpr int64_t WIN_MAX_BINS = 32768;   // histogram bins (132 KB of shared memory in the cuts)
+// output room reserved from the bound on the terms up to this many bytes; above
+// it the distinct keys are estimated first
+constexpr double WIN_BOUND_BYTES = 16.0 * 1024 * 1024 * 1024;
 constexpr int HASH_TILE_I = 32;
 constexpr int HASH_TILE_J = 1024;
 
