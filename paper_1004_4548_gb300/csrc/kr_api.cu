@@ -899,10 +899,12 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     ck(ctx, cudaMemsetAsync(Z.zero, 0, Z.zero_bytes, s), "memset accumulators");
     mark(ctx, s, "zero_accumulators");
     if (!dense_ids.empty()) {
+      bool clipped = false;
+      for (int p : dense_ids) clipped |= plans[p].p.clip != 0;
       ck(ctx, launch_dense_plan(A.lprods, A.dense_ids, A.block_begin, (int)dense_ids.size(),
-                                nblocks_total, A.tasks, dense_tasks_total, Z.counters, s),
+                                nblocks_total, clipped, A.tasks, dense_tasks_total, Z.counters, s),
          "dense plan");
-      ctx->launches += 1;
+      ctx->launches += clipped ? 2 : 1;
       mark(ctx, s, "dense_plan");
       ck(ctx, launch_dense_accum(A.lprods, A.tasks, Z.counters, dense_tasks_total, Z.counters + 1,
                                  ctx->num_sms, max_S, s),

@@ -17,99 +17,197 @@
 
 namespace kr {
 
-constexpr int PLAN_SAMPLES = 32;   // sampled i per block for the work estimate
 constexpr int MAX_SPLIT = 64;      // tasks per block at most
+constexpr int PLAN_THREADS = 256;
+constexpr int PLAN_PER = 8;        // f terms looked at per planning thread
+constexpr int PLAN_TERM_COST = 8;  // an f term examined costs about as much as this many pairs
 constexpr int ACC_THREADS = 512;
 
-// One warp per (dense product, block): i-range by warp-wide search, sampled
-// work estimate, then 1..MAX_SPLIT tasks over equal i-slices.  A block that
-// gets one task is written whole by its flush; every other block (several
-// tasks adding into it, or none) is zeroed here, so the accumulation array
-// needs no separate clearing.
-__global__ void __launch_bounds__(256) k_dense_plan(const Prod* __restrict__ prods,
-                                                   const int32_t* __restrict__ dense_prods,
-                                                   const int64_t* __restrict__ block_begin,
-                                                   int ndense, DenseTask* __restrict__ tasks,
-                                                   int64_t task_cap, int64_t* __restrict__ task_count) {
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t total = block_begin[ndense];
-  if (gw >= total) return;
-  // product owning global block gw
-  int lo = 0, hi = ndense - 1;
+// The f terms that reach an output block, and about how many g terms pair with
+// them into it: every st-th term of [i_lo, i_hi), PLAN_PER consecutive ones per
+// thread, counted by the g bucket index alone (both ends rounded down to their
+// bucket, so the counts are right on average).
+struct BlockWork {
+  int64_t B, E;          // the block's codes
+  int64_t i_lo, i_hi, st;
+  int pid;
+  int64_t b;             // block of the product
+  int32_t cnt[PLAN_PER]; // work of the looked-at terms: their pairs and the cost of examining them
+  int64_t sum;           // of this thread's
+};
+
+// false: nothing to do (no such block).  By a whole CTA; s_range: two words.
+__device__ __forceinline__ bool block_work(const Prod* prods, const int32_t* dense_prods, const int64_t* block_begin,
+                                           int ndense, int64_t* s_range, BlockWork& W) {
+  const int64_t gw = blockIdx.x;
+  if (gw >= block_begin[ndense]) return false;
+  int lo = 0, hi = ndense - 1;   // product owning global block gw
   while (lo < hi) {
     int mid = (lo + hi + 1) >> 1;
     if (block_begin[mid] <= gw) lo = mid; else hi = mid - 1;
   }
-  const int pid = dense_prods[lo];
-  const Prod& P = prods[pid];
-  const int64_t b = gw - block_begin[lo];
+  W.pid = dense_prods[lo];
+  const Prod& P = prods[W.pid];
+  W.b = gw - block_begin[lo];
   // blocks tile the key window [klo, klo + kspan); its end may fall inside the last block
-  const int64_t B = P.klo + b * P.S, E = min(B + P.S, P.klo + P.kspan);
-  int64_t k = 0;
+  W.B = P.klo + W.b * P.S;
+  W.E = min(W.B + P.S, P.klo + P.kspan);
   const int64_t* F = P.f.code;
   const int64_t* G = P.g.code;
   const int64_t nf = P.f.nkeep, ng = P.g.nkeep;   // dropped terms sort last
-  if (!P.status && nf > 0 && ng > 0) {
-    int64_t i_lo, i_hi;
-    warp_lower_bound2(F, nf, B - G[ng - 1], E - G[0], &i_lo, &i_hi);
-    if (i_lo < i_hi) {
-      const int32_t* gx = P.gidx;
-      const int64_t gn = P.gidx_n;
-      const int gsh = P.gshift;
-      const int64_t span = i_hi - i_lo;
-      int64_t cnt = 0;
-      const int ns = span < PLAN_SAMPLES ? (int)span : PLAN_SAMPLES;
-      if (lane < ns) {
-        const int64_t i = i_lo + (span * lane) / ns;
-        int64_t a, c;
-        g_lower_bound2(G, ng, gx, gn, gsh, B - F[i], E - F[i], &a, &c);
-        cnt = c - a;
+  if (threadIdx.x < 32) {
+    int64_t a = 0, c = 0;
+    if (!P.status && nf > 0 && ng > 0) warp_lower_bound2(F, nf, W.B - G[ng - 1], W.E - G[0], &a, &c);
+    if (threadIdx.x == 0) {
+      s_range[0] = a;
+      s_range[1] = c;
+    }
+  }
+  __syncthreads();
+  W.i_lo = s_range[0];
+  W.i_hi = s_range[1];
+  const int64_t span = W.i_hi - W.i_lo;
+  W.st = max((int64_t)1, (span + PLAN_THREADS * PLAN_PER - 1) / (PLAN_THREADS * PLAN_PER));
+  W.sum = 0;
+  int64_t a[PLAN_PER];
+#pragma unroll
+  for (int q = 0; q < PLAN_PER; ++q) {
+    const int64_t i = W.i_lo + ((int64_t)threadIdx.x * PLAN_PER + q) * W.st;
+    a[q] = i < W.i_hi ? F[i] : -1;   // codes are never negative
+  }
+#pragma unroll
+  for (int q = 0; q < PLAN_PER; ++q) {
+    W.cnt[q] = 0;
+    if (a[q] >= 0) {
+      auto below = [&](int64_t x) -> int64_t {
+        const int64_t k = x >> P.gshift;
+        return x <= 0 ? 0 : k >= P.gidx_n ? ng : min((int64_t)P.gidx[k], ng);
+      };
+      W.cnt[q] = (int32_t)(below(W.E - a[q]) - below(W.B - a[q])) + PLAN_TERM_COST;
+    }
+    W.sum += W.cnt[q];
+  }
+  return true;
+}
+
+// Work of every clipped product (truncated, or a key window), which its tasks
+// are sized by (of an unclipped one the number of pairs is known).
+__global__ void __launch_bounds__(PLAN_THREADS) k_dense_work(Prod* __restrict__ prods,
+                                                             const int32_t* __restrict__ dense_prods,
+                                                             const int64_t* __restrict__ block_begin, int ndense) {
+  __shared__ int64_t s_range[2];
+  BlockWork W;
+  if (!block_work(prods, dense_prods, block_begin, ndense, s_range, W)) return;
+  Prod& P = prods[W.pid];
+  if (P.work_target > 0) return;
+  int64_t x = W.sum * W.st;
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if ((threadIdx.x & 31) == 0 && x) atomicAdd(&P.work, (unsigned long long)x);
+}
+
+// One CTA per (dense product, block): the block's work split into 1..MAX_SPLIT
+// tasks of equal work over consecutive f terms.  (Equal numbers of f terms per
+// task, by 32 sampled terms a block, left the slowest CTA three times the mean
+// on a truncated product and twice on a 9.4 M pair one.)  Accumulation on GB300:
+// 14950 x 14950 terms truncated at their degree 120 -> 60 us, 4384 x 2153
+// float64 terms 179 -> 109 us, 46376 x 46376 terms 3.15 -> 2.90 ms.  A block
+// that gets one task is written whole by its flush; every other block (several
+// tasks adding into it, or none) is zeroed here, so the accumulation array needs
+// no separate clearing.
+__global__ void __launch_bounds__(PLAN_THREADS) k_dense_plan(const Prod* __restrict__ prods,
+                                                             const int32_t* __restrict__ dense_prods,
+                                                             const int64_t* __restrict__ block_begin, int ndense,
+                                                             DenseTask* __restrict__ tasks, int64_t task_cap,
+                                                             int64_t* __restrict__ task_count) {
+  __shared__ int64_t s_range[2], s_warp[PLAN_THREADS / 32], s_cut[MAX_SPLIT + 1], s_th[MAX_SPLIT], s_base, s_target;
+  BlockWork W;
+  if (!block_work(prods, dense_prods, block_begin, ndense, s_range, W)) return;
+  const Prod& P = prods[W.pid];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t span = W.i_hi - W.i_lo;
+  int64_t k = 0;
+  if (span > 0) {   // uniform
+    const int64_t mine = W.sum;
+    int64_t x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    if (tid == 0) {
+      const int64_t t = P.work_target > 0 ? P.work_target : dense_work_target((double)P.work, (double)P.ctas, P.S);
+      // the tasks' sizes fall along the queue, which the blocks enter in order, so
+      // that the last ones are short (10626 x 10626 terms: 194 us against 217
+      // with tasks of one size)
+      s_target = max((int64_t)1, (int64_t)((float)t * (2.0f - 1.6f * (float)W.b / (float)P.nblocks)));
+    }
+    __syncthreads();
+    int64_t before = x - mine, total = 0;
+    for (int w = 0; w < PLAN_THREADS / 32; ++w) {
+      if (w < warp) before += s_warp[w];
+      total += s_warp[w];
+    }
+    // a zero estimate does not prove an empty block (the terms between the
+    // looked-at ones may pair), so every block with a nonempty i-range gets at
+    // least one task
+    k = min(min(total * W.st / s_target + 1, (int64_t)MAX_SPLIT), span);
+    // cut t: after the first looked-at term that takes the work to the t-th threshold
+    if (tid == 0) s_cut[0] = W.i_lo;
+    else if (tid < k) s_th[tid] = total * tid / k;
+    __syncthreads();
+    int lo = 1, hi = (int)k;   // the first threshold past the work before this thread's terms
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (s_th[mid] > before) hi = mid; else lo = mid + 1;
+    }
+    int64_t c = before;
+#pragma unroll
+    for (int q = 0; q < PLAN_PER; ++q) {
+      const int64_t i = W.i_lo + ((int64_t)tid * PLAN_PER + q) * W.st;
+      if (i < W.i_hi) {
+        c += W.cnt[q];
+        for (; lo < k && s_th[lo] <= c; ++lo) s_cut[lo] = min(i + W.st, W.i_hi);
       }
-      for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-      // a zero estimate does not prove an empty block (the samples may all miss),
-      // so every block with a nonempty i-range gets at least one task
-      const double est = (double)cnt * (double)span / (double)ns;
-      k = (int64_t)(est / (double)P.work_target) + 1;
-      if (k > MAX_SPLIT) k = MAX_SPLIT;
-      if (k > span) k = span;
-      int64_t base = 0;
-      if (lane == 0) base = (int64_t)atomicAdd((unsigned long long*)task_count, (unsigned long long)k);
-      base = __shfl_sync(0xffffffffu, base, 0);
-      for (int64_t t = lane; t < k; t += 32) {
-        if (base + t >= task_cap) break;
-        DenseTask T;
-        T.prod = pid;
-        T.pad = 0;
-        T.block = b;
-        T.i0 = i_lo + (span * t) / k;
-        T.i1 = i_lo + (span * (t + 1)) / k;
-        T.single = (k == 1);
-        tasks[base + t] = T;
-      }
+    }
+    if (tid == 0) {
+      s_cut[k] = W.i_hi;
+      s_base = (int64_t)atomicAdd((unsigned long long*)task_count, (unsigned long long)k);
+    }
+    __syncthreads();
+    for (int64_t t = tid; t < k; t += PLAN_THREADS) {
+      if (s_base + t >= task_cap) break;
+      DenseTask T;
+      T.prod = W.pid;
+      T.pad = 0;
+      T.block = W.b;
+      T.i0 = s_cut[t];
+      T.i1 = s_cut[t + 1];
+      T.single = (k == 1);
+      tasks[s_base + t] = T;
     }
   }
   if (k != 1 && P.dense) {
     // 16-byte stores over the block's slots, with an 8-byte store for a slot
     // before the first 16-byte boundary and for an unpaired last slot
-    uint64_t* out = (uint64_t*)P.dense + (B - P.klo);
-    const int64_t len = E - B;
+    uint64_t* out = (uint64_t*)P.dense + (W.B - P.klo);
+    const int64_t len = W.E - W.B;
     const int64_t head = ((uintptr_t)out & 15) ? 1 : 0;
-    if (head && lane == 0 && len > 0) out[0] = 0;
-    for (int64_t s = head + 2 * lane; s + 1 < len; s += 64) *(uint4*)(out + s) = make_uint4(0, 0, 0, 0);
-    if (len > head && ((len - head) & 1) && lane == 0) out[len - 1] = 0;
+    if (head && tid == 0 && len > 0) out[0] = 0;
+    for (int64_t s = head + 2 * tid; s + 1 < len; s += 2 * PLAN_THREADS) *(uint4*)(out + s) = make_uint4(0, 0, 0, 0);
+    if (len > head && ((len - head) & 1) && tid == 0) out[len - 1] = 0;
   }
 }
 
-cudaError_t launch_dense_plan(const Prod* dprods, const int32_t* ddense_prods,
-                              const int64_t* dblock_begin, int ndense, int64_t nblocks_total,
+cudaError_t launch_dense_plan(Prod* dprods, const int32_t* ddense_prods,
+                              const int64_t* dblock_begin, int ndense, int64_t nblocks_total, bool clipped,
                               DenseTask* dtasks, int64_t task_cap, int64_t* dtask_count,
                               cudaStream_t s) {
   if (nblocks_total <= 0) return cudaSuccess;
-  const int64_t threads = nblocks_total * 32;
-  const int64_t grid = (threads + 255) / 256;
-  k_dense_plan<<<(unsigned)grid, 256, 0, s>>>(dprods, ddense_prods, dblock_begin, ndense, dtasks,
-                                              task_cap, dtask_count);
+  if (clipped)
+    k_dense_work<<<(unsigned)nblocks_total, PLAN_THREADS, 0, s>>>(dprods, ddense_prods, dblock_begin, ndense);
+  k_dense_plan<<<(unsigned)nblocks_total, PLAN_THREADS, 0, s>>>(dprods, ddense_prods, dblock_begin, ndense, dtasks,
+                                                                task_cap, dtask_count);
   return cudaGetLastError();
 }
 

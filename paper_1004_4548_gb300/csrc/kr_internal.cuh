@@ -207,7 +207,9 @@ struct Prod {
   // dense path
   int64_t S;            // output codes per block
   int64_t nblocks;
-  int64_t work_target;  // pairs per task
+  int64_t work_target;  // work per task (pairs); 0: from the device's estimate (work) of a clipped product
+  int64_t ctas;         // accumulating CTAs resident at once
+  unsigned long long work;
   void* dense;          // [kspan] accumulators (slot = key - klo)
   int32_t* gidx;        // gidx[b] = first j with g.code[j] >= b << gshift, b in [0, gidx_n]
   int64_t gidx_n;       // buckets (the last entry gidx[gidx_n] = g.n)
@@ -468,8 +470,24 @@ cudaError_t launch_harmonic_pack(Prod* dprods, const OpRef* dops, int nops, int6
 cudaError_t launch_mag_keys(Prod* dprods, const OpRef* dops, int nops, int64_t max_n, cudaStream_t s);
 cudaError_t launch_mag_reorder(Prod* dprods, const OpRef* dops, int nops, int64_t max_n, cudaStream_t s);
 
-cudaError_t launch_dense_plan(const Prod* dprods, const int32_t* ddense_prods,
-                              const int64_t* dblock_begin, int ndense, int64_t nblocks_total,
+// Pairs per task of a dense product: between two and six tasks per resident CTA
+// for products of 2e4 to 6e4 pairs per CTA (the task queue evens out what the
+// estimates miss; more tasks cost more clearing and flushing of slices), more
+// for larger ones (tasks of about 50,000 pairs, at most 24 per CTA, so that the
+// last ones, which set the run's tail, stay short), and no task below half a
+// pair per slice slot.
+__host__ __device__ inline int64_t dense_work_target(double pairs, double ctas, int64_t S) {
+  double per_cta = pairs / (ctas * 1e4);
+  per_cta = per_cta < 2.0 ? 2.0 : per_cta > 6.0 ? 6.0 : per_cta;
+  double more = pairs / (ctas * 5e4);
+  more = more > 24.0 ? 24.0 : more;
+  if (more > per_cta) per_cta = more;
+  const double tgt = pairs / (ctas * per_cta), least = 0.5 * (double)S;
+  return (int64_t)(tgt > least ? tgt : least) + 1;
+}
+// clipped: some product is truncated or a key window (its pairs are counted first)
+cudaError_t launch_dense_plan(Prod* dprods, const int32_t* ddense_prods,
+                              const int64_t* dblock_begin, int ndense, int64_t nblocks_total, bool clipped,
                               DenseTask* dtasks, int64_t task_cap, int64_t* dtask_count,
                               cudaStream_t s);
 cudaError_t launch_build_gindex(const Prod* dprods, const int32_t* ddense_prods, int ndense,

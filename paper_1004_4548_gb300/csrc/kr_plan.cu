@@ -4,12 +4,6 @@
 
 #include "kr_plan.h"
 
-// dense path: tasks per resident CTA (more: a shorter tail of the dynamic
-// task queue; fewer: less zeroing and flushing of block slices)
-#ifndef KR_TASKS_PER_CTA
-#define KR_TASKS_PER_CTA 6
-#endif
-
 namespace kr {
 
 int bits_for(uint64_t range) {
@@ -320,20 +314,16 @@ void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_
     if (S > kr32) S = kr32;
     P.S = S;
     P.nblocks = ceil_div(P.kspan, S);
-    // ~6 tasks per resident CTA so the dynamic task queue evens out the
-    // uneven (diamond-shaped) work per output block
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(4, (227 * 1024) / (S * 8 + 11264)));
-    // tasks per resident CTA: at least KR_TASKS_PER_CTA, more for large
-    // products (tasks of about 50,000 term-products, at most 24 per CTA), so
-    // that the last tasks, which set the run's tail, stay short
-    const double ctas = (double)num_sms * (double)per_sm;
-    const double per_cta = std::min(24.0, std::max((double)KR_TASKS_PER_CTA, pairs / (ctas * 5e4)));
-    const double tgt = pairs / (ctas * per_cta);
-    P.work_target = (int64_t)std::max(tgt, (double)(2 * S));
+    P.ctas = num_sms * per_sm;
+    P.work_target = P.clip ? 0 : dense_work_target(pairs, (double)P.ctas, S);
     pl.dense_task_cap = P.nblocks * 64;
-    // bucket index over g's codes: at most 65536 buckets
+    // bucket index over g's codes: at most 65536 buckets, and a few per term (a
+    // bucket costs a store, and small products have few threads for them: 48,000
+    // buckets of 1001 terms took 27 us of a 0.15 ms call)
     int sh = 0;
-    while (((P.g.key_range >> sh) + 1) > 65535) ++sh;
+    const int64_t most = std::min<int64_t>(65535, std::max<int64_t>(256, 8 * ng));
+    while (((P.g.key_range >> sh) + 1) > most) ++sh;
     P.gshift = sh;
     P.gidx_n = (P.g.key_range >> sh) + 1;
     pl.accum_bytes = P.kspan * 8;

@@ -148,7 +148,8 @@ extern "C" kr_status kron_dense_product_static(const int64_t* fcode, const void*
   P.S = S;
   P.nblocks = nblocks;
   const double pairs = (double)nf * (double)ng;
-  P.work_target = (int64_t)std::max(pairs / (double)(sms * 4), (double)(2 * S));
+  P.ctas = 3 * sms;   // 64 KB slices
+  P.work_target = dense_work_target(pairs, (double)P.ctas, S);
   P.dense = out;
   P.gidx = (int32_t*)(base + off_gidx);
   P.gidx_n = gidx_n;
@@ -168,7 +169,7 @@ extern "C" kr_status kron_dense_product_static(const int64_t* fcode, const void*
   k_static_check<<<(unsigned)check_blocks, 256, 0, s>>>(dprod, W);
   if (cudaGetLastError() != cudaSuccess) return KR_ERR_CUDA;
   if (launch_build_gindex(dprod, dsmall->ids, 1, ng, s) != cudaSuccess ||
-      launch_dense_plan(dprod, dsmall->ids, dsmall->block_begin, 1, nblocks, dtasks, task_cap, dcnt, s) !=
+      launch_dense_plan(dprod, dsmall->ids, dsmall->block_begin, 1, nblocks, false, dtasks, task_cap, dcnt, s) !=
           cudaSuccess) {
     cudaGetLastError();
     return KR_ERR_CUDA;
