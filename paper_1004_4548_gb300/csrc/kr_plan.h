@@ -36,6 +36,7 @@ constexpr int DEFAULT_PROBES = 512;
 // searches that find nothing)
 constexpr int64_t WIN_MAX_LIST = int64_t(1) << 20;
 constexpr double WIN_MAX_WALK = 65536.0;
+constexpr int64_t WIN_MIN_ARRAY = int64_t(1) << 24;   // keys of an array of L2's size (128 MB)
 constexpr int64_t WIN_MAX_BINS = 32768;   // histogram bins (132 KB of shared memory in the cuts)
 // output room reserved from the bound on the terms up to this many bytes; above
 // it the distinct keys are estimated first
