@@ -67,6 +67,16 @@ struct kr_ctx {
   const uint64_t* res_val = nullptr;
   int64_t res_n = 0;                    // -1 until a deferred count is read
   const int64_t* res_err = nullptr;     // deferred: the compaction's wait error word
+  // a windowed product whose windows have not been put together: its decode
+  // does that (allow_raw: the call's outputs are those of a single product);
+  // raw_key / raw_val: room for its ordered terms, for the outputs that need them
+  bool allow_raw = false;
+  bool res_raw = false;
+  WinLaunch raw{};
+  int64_t raw_cap = 0;
+  uint64_t* raw_key = nullptr;
+  uint64_t* raw_val = nullptr;
+  int64_t* raw_total = nullptr;
   // stage timing (CUDA events on the call's stream) and launch counting
   bool profile = false;
   std::vector<cudaEvent_t> ev;
@@ -946,13 +956,32 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     for (int k = 0, at = 0; k < 2; at += (int)win_ids[k].size(), ++k) {
       if (win_ids[k].empty()) continue;
       int wl = 0;
-      ck(ctx, launch_window(A.lprods, A.win_ids + at, A.win_prefix[k], (int)win_ids[k].size(), k + 1,
-                            k ? win_cap_total - win_cap_total1 : win_cap_total1, Z.counters + 4 + k, Z.wout[k],
-                            Z.wbefore, Z.wscan, wbase, Z.wtotal + k, out_total, Z.okey, Z.oval, Z.wstage,
-                            win_stage, ctx->num_sms, s, &wl),
+      WinLaunch L;
+      L.prods = A.win_ids + at;
+      L.rprefix = A.win_prefix[k];
+      L.nwp = (int)win_ids[k].size();
+      L.kind = k + 1;
+      L.max_windows = k ? win_cap_total - win_cap_total1 : win_cap_total1;
+      L.out = Z.wout[k];
+      L.before = Z.wbefore;
+      L.scan = Z.wscan;
+      ck(ctx, launch_window(A.lprods, L, Z.counters + 4 + k, Z.wstage, win_stage, ctx->num_sms, s, &wl),
          "window accumulate");
-      wbase = Z.wtotal + k;
       ctx->launches += wl;
+      if (ctx->allow_raw && nprod == 1 && !ctx->replay) {
+        // the only product: its decode puts the windows together
+        ctx->raw = L;
+        ctx->raw_cap = out_total;
+        ctx->raw_key = Z.okey;
+        ctx->raw_val = Z.oval;
+        ctx->raw_total = Z.wtotal + k;
+        ctx->res_raw = true;
+      } else {
+        ck(ctx, launch_win_copy(A.lprods, L, wbase, Z.wtotal + k, out_total, Z.okey, Z.oval, ctx->num_sms, s),
+           "window copy");
+        ctx->launches += 1;
+        wbase = Z.wtotal + k;
+      }
       mark(ctx, s, "hash_insert");
     }
     if (deferred) {
@@ -1112,6 +1141,24 @@ void copy_out(kr_ctx* ctx, void* dst, const void* src, size_t bytes, cudaStream_
 
 kr_status settle_deferred(kr_ctx* ctx, cudaStream_t s);
 
+// The kept product's windows decoded into the caller's device arrays.
+void decode_raw(kr_ctx* ctx, bool series, const SeriesOut& out, cudaStream_t s) {
+  ck(ctx, launch_win_decode(ctx->res_dprod, ctx->raw, series, out, ctx->num_sms, s), "window decode");
+  ctx->launches += 1;
+  mark(ctx, s, "decode");
+}
+
+// The kept product's windows put together in the context's own arrays.
+void join_raw(kr_ctx* ctx, cudaStream_t s) {
+  if (!ctx->res_raw) return;
+  ck(ctx, launch_win_copy(ctx->res_dprod, ctx->raw, nullptr, ctx->raw_total, ctx->raw_cap, ctx->raw_key, ctx->raw_val,
+                          ctx->num_sms, s), "window copy");
+  ctx->launches += 1;
+  ctx->res_key = ctx->raw_key;
+  ctx->res_val = ctx->raw_val;
+  ctx->res_raw = false;
+}
+
 kr_status emit_poly(kr_ctx* ctx, kr_poly_out* h, cudaStream_t s) {
   const Prod& P = ctx->res_prod;
   const int64_t n = ctx->res_n;
@@ -1132,6 +1179,23 @@ kr_status emit_poly(kr_ctx* ctx, kr_poly_out* h, cudaStream_t s) {
     h->nterms = st == KR_OK ? ctx->res_n : 0;
     if (st != KR_OK) return st;
     return ctx->res_n > h->capacity ? KR_ERR_CAPACITY : KR_OK;
+  }
+  if (ctx->res_raw) {
+    if (is_device_ptr(h->coef) && (!h->exps || is_device_ptr(h->exps)) && (!h->codes || is_device_ptr(h->codes))) {
+      if (n > h->capacity) return KR_ERR_CAPACITY;
+      if (n == 0) return KR_OK;
+      decode_raw(ctx, false, SeriesOut{h->exps, nullptr, nullptr, h->codes, (uint64_t*)h->coef, h->capacity}, s);
+      if (n > 0) {
+        ck(ctx, cudaStreamSynchronize(s), "sync output");
+        collect_stages(ctx);
+        return KR_OK;
+      }
+      const kr_status st = settle_deferred(ctx, s);
+      h->nterms = st == KR_OK ? ctx->res_n : 0;
+      if (st != KR_OK) return st;
+      return ctx->res_n > h->capacity ? KR_ERR_CAPACITY : KR_OK;
+    }
+    join_raw(ctx, s);
   }
   if (n < 0) {
     const bool exps_dev = !h->exps || is_device_ptr(h->exps);
@@ -1219,6 +1283,22 @@ kr_status emit_pseries(kr_ctx* ctx, kr_pseries_out* h, cudaStream_t s) {
   const Prod& P = ctx->res_prod;
   const int64_t n = ctx->res_n;
   h->nterms = n;
+  const bool all_dev = is_device_ptr(h->coef) && (!h->exps || is_device_ptr(h->exps)) &&
+                       (!h->trig || is_device_ptr(h->trig)) && (!h->kind || is_device_ptr(h->kind)) &&
+                       (!h->codes || is_device_ptr(h->codes));
+  if (ctx->res_raw && all_dev && n != 0 && n <= h->capacity) {
+    decode_raw(ctx, true, SeriesOut{h->exps, h->trig, h->kind, h->codes, (uint64_t*)h->coef, h->capacity}, s);
+    if (n > 0) {
+      ck(ctx, cudaStreamSynchronize(s), "sync output");
+      collect_stages(ctx);
+      return KR_OK;
+    }
+    const kr_status st = settle_deferred(ctx, s);
+    h->nterms = st == KR_OK ? ctx->res_n : 0;
+    if (st != KR_OK) return st;
+    return ctx->res_n > h->capacity ? KR_ERR_CAPACITY : KR_OK;
+  }
+  if (ctx->res_raw && n <= h->capacity) join_raw(ctx, s);
   if (n < 0) {
     // deferred count (device outputs only), as in emit_poly
     ck(ctx, launch_decode_pseries(ctx->res_dprod, 0, ctx->res_key, h->capacity, h->exps, h->trig, h->kind,
@@ -1539,6 +1619,8 @@ kr_status poly_mul(kr_ctx* ctx, const kr_poly* f, const kr_poly* g, kr_poly_out*
     // until the decode into scratch, whose terms are then copied); with every
     // output in device memory the compaction may decode into it directly
     ctx->allow_deferred = true;
+    ctx->allow_raw = true;
+    ctx->res_raw = false;
     ctx->direct = DirectOut{};
     ctx->direct_done = false;
     if (h->capacity > 0) {
@@ -1558,12 +1640,12 @@ kr_status poly_mul(kr_ctx* ctx, const kr_poly* f, const kr_poly* g, kr_poly_out*
     try {
       run_pipeline(ctx, {in}, s, res);
     } catch (...) {
-      ctx->allow_deferred = false;
+      ctx->allow_deferred = ctx->allow_raw = false;
       ctx->direct = DirectOut{};
       ctx->direct_done = false;
       throw;
     }
-    ctx->allow_deferred = false;
+    ctx->allow_deferred = ctx->allow_raw = false;
     ctx->direct = DirectOut{};
     if (res[0].st != KR_OK) {
       ctx->direct_done = false;
@@ -1611,15 +1693,17 @@ kr_status poisson_mul(kr_ctx* ctx, const kr_pseries* f, const kr_pseries* g, kr_
     ctx->allow_deferred = is_device_ptr(h->coef) && (!h->exps || is_device_ptr(h->exps)) &&
                           (!h->trig || is_device_ptr(h->trig)) && (!h->kind || is_device_ptr(h->kind)) &&
                           (!h->codes || is_device_ptr(h->codes));
+    ctx->allow_raw = true;
+    ctx->res_raw = false;
     ctx->direct = DirectOut{};
     ctx->direct_done = false;
     try {
       run_pipeline(ctx, {in}, s, res);
     } catch (...) {
-      ctx->allow_deferred = false;
+      ctx->allow_deferred = ctx->allow_raw = false;
       throw;
     }
-    ctx->allow_deferred = false;
+    ctx->allow_deferred = ctx->allow_raw = false;
     if (res[0].st != KR_OK) return res[0].st;
     keep_result(ctx, res[0], true);
     return emit_pseries(ctx, h, s);

@@ -564,7 +564,8 @@ __global__ void __launch_bounds__(256) k_decode_poly(const Prod* __restrict__ pr
                                                      int64_t* __restrict__ codes, int dev_count,
                                                      const uint64_t* __restrict__ vals,
                                                      uint64_t* __restrict__ coef) {
-  const Prod& P = prods[prod];
+  __shared__ Prod s_prod;
+  const Prod& P = shared_prod(&prods[prod], &s_prod);
   if (dev_count) n = P.status ? 0 : min(n, P.nout);
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -595,7 +596,8 @@ __global__ void __launch_bounds__(256) k_decode_pseries(const Prod* __restrict__
                                                         int64_t* __restrict__ codes, int dev_count,
                                                         const uint64_t* __restrict__ vals,
                                                         uint64_t* __restrict__ coef) {
-  const Prod& P = prods[prod];
+  __shared__ Prod s_prod;
+  const Prod& P = shared_prod(&prods[prod], &s_prod);
   if (dev_count) n = P.status ? 0 : min(n, P.nout);
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
@@ -643,15 +645,10 @@ __global__ void __launch_bounds__(256) k_decode_batch(const Prod* __restrict__ p
       const int64_t per_kind = P.T2 * P.Wp;
       const int64_t kd = key >= per_kind ? 1 : 0;   // keys lie below 2 * per_kind
       int64_t pc;
-      const int64_t T = divmod_nn(key - kd * per_kind, P.Wp, &pc);
+      const int64_t T = divmod(key - kd * per_kind, P.divWp, &pc);
       R.kind[t] = (uint8_t)kd;
       if (P.np > 0) decode_poly_part(P, pc, R.exps, R.n, t);
-      int64_t u = T + (P.T2 - 1);
-      for (int k = 0; k < P.nt; ++k) {
-        int64_t d = u;
-        if (k + 1 < P.nt) u = divmod_nn(u, P.w[P.np + k], &d);
-        R.trig[(int64_t)k * R.n + t] = (int32_t)(d + P.omin[P.np + k]);
-      }
+      decode_digits(P.div + P.np, P.omin + P.np, P.nt, T + (P.T2 - 1), R.trig + t, R.n);
     }
   }
 }
@@ -674,6 +671,7 @@ struct Box {
   int32_t emin[MAXV];
   int32_t emax[MAXV];
   int32_t w[MAXV];
+  Divisor div[MAXV];
   int64_t c[MAXV];
 };
 
@@ -700,22 +698,19 @@ __global__ void k_decode_box(const int64_t* __restrict__ codes, int64_t n, int n
        i += (int64_t)gridDim.x * blockDim.x) {
     int64_t rem = codes[i];
     if (rem < 0 || rem >= W) { bad = 1; rem = 0; }
-    for (int k = 0; k < nvars; ++k) {
-      int64_t d = rem;
-      if (k + 1 < nvars) rem = divmod_nn(rem, b.w[k], &d);
-      exps[(int64_t)k * n + i] = (int32_t)(d + b.emin[k]);
-    }
+    decode_digits(b.div, b.emin, nvars, rem, exps + i, n);
   }
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, ST_RANGE);
 }
 
 static Box make_box(int nvars, const int32_t* emin, const int32_t* emax, const int64_t* cvec) {
   Box b;
-  for (int k = 0; k < MAXV; ++k) { b.emin[k] = 0; b.emax[k] = 0; b.w[k] = 1; b.c[k] = 0; }
+  for (int k = 0; k < MAXV; ++k) { b.emin[k] = 0; b.emax[k] = 0; b.w[k] = 1; b.c[k] = 0; b.div[k] = make_divisor(1); }
   for (int k = 0; k < nvars; ++k) {
     b.emin[k] = emin[k];
     b.emax[k] = emax[k];
     b.w[k] = emax[k] - emin[k] + 1;
+    b.div[k] = make_divisor(b.w[k]);
     b.c[k] = cvec[k];
   }
   return b;

@@ -161,6 +161,22 @@ struct Win {
   double* bcoef;         // Poisson: [2 nb]
 };
 
+// A divisor with its reciprocals: floor(2^32 / d) (at most 2^32 - 1) and
+// floor((2^64 - 1) / d).
+struct Divisor {
+  int64_t d;
+  uint64_t r64;
+  uint32_t r32;
+};
+inline Divisor make_divisor(int64_t d) {
+  Divisor v;
+  v.d = d;
+  v.r64 = ~0ull / (uint64_t)d;
+  const uint64_t r = (uint64_t(1) << 32) / (uint64_t)d;
+  v.r32 = r > 0xffffffffull ? 0xffffffffu : (uint32_t)r;
+  return v;
+}
+
 // One product, planned on the host, read by every kernel.
 struct Prod {
   Operand f, g;
@@ -170,6 +186,8 @@ struct Prod {
   int32_t coef32;       // int64 coefficients that all fit in int32 (32x32->64 multiply)
   int64_t c[MAXV];      // coding vector; poly part [0, np), trig part [np, np + nt)
   int32_t w[MAXV];      // output widths
+  Divisor div[MAXV];    // the same, to divide by
+  Divisor divWp;        // and the polynomial code range
   int32_t omin[MAXV];   // output box minimum (poly), -R_k (trig)
   // truncated product (graded coding): the degree in the variables of gmask
   // replaces variable gvar and is the most significant polynomial digit; the
@@ -323,18 +341,60 @@ __device__ __forceinline__ void g_lower_bound2(const int64_t* G, int64_t ng, con
   *r2 = lo2;
 }
 
-// q = x / d and *r = x % d for x >= 0, d >= 1: 32-bit division when x fits
-// (a 64-bit division costs several times more), which after the first digits
-// of a code is almost always the case.
-__device__ __forceinline__ int64_t divmod_nn(int64_t x, int64_t d, int64_t* r) {
-  if ((uint64_t)x <= 0xffffffffull && d <= 0xffffffffll) {
-    const uint32_t q = (uint32_t)x / (uint32_t)d;
-    *r = (int64_t)((uint32_t)x - q * (uint32_t)d);
+// q = x / d and *r = x % d for 0 <= x < 2^63, d >= 1: the reciprocal's product
+// is at most one below the quotient (the reciprocal is less than one below
+// 2^32 / d, or 2^64 / d, and x is below 2^32, or 2^63), so one comparison
+// mends it.  A digit takes 5 instructions where x fits 32 bits, which after the
+// first digits of a code it nearly always does, and about 20 otherwise, against
+// about 20 and 80 for a plain division (3 million codes of five digits decoded,
+// the call with its encoding: 146 -> 120 us).
+__device__ __forceinline__ int64_t divmod(int64_t x, const Divisor& v, int64_t* r) {
+  if ((uint64_t)x <= 0xffffffffull && (uint64_t)v.d <= 0xffffffffull) {
+    const uint32_t n = (uint32_t)x, d = (uint32_t)v.d;
+    uint32_t q = __umulhi(n, v.r32), m = n - q * d;
+    if (m >= d) { ++q; m -= d; }
+    *r = m;
     return q;
   }
-  const int64_t q = x / d;
-  *r = x - q * d;
-  return q;
+  uint64_t q = __umul64hi((uint64_t)x, v.r64), m = (uint64_t)x - q * (uint64_t)v.d;
+  if (m >= (uint64_t)v.d) { ++q; m -= (uint64_t)v.d; }
+  *r = (int64_t)m;
+  return (int64_t)q;
+}
+
+// A product's plan copied to shared memory by the CTA: the decoding kernels read
+// a few words of it per digit, which as global loads are repeated after every
+// store (the compiler cannot tell that the outputs do not overlap it).
+__device__ __forceinline__ const Prod& shared_prod(const Prod* p, Prod* copy) {
+  static_assert(sizeof(Prod) % 8 == 0, "copied by 8-byte words");
+  for (int i = threadIdx.x; i < (int)(sizeof(Prod) / 8); i += blockDim.x)
+    ((uint64_t*)copy)[i] = ((const uint64_t*)p)[i];
+  __syncthreads();
+  return *copy;
+}
+
+// Mixed-radix digits of x (n of them, least significant first, digit k plus
+// lo[k]) to p[0], p[ld], ...: in 32 bits as soon as what is left of x fits.
+__device__ __forceinline__ void decode_digits(const Divisor* div, const int32_t* lo, int n, int64_t x,
+                                              int32_t* __restrict__ p, int64_t ld) {
+  int k = 0;
+  while (k + 1 < n && (uint64_t)x >> 32) {
+    int64_t d;
+    x = divmod(x, div[k], &d);
+    *p = (int32_t)(d + lo[k]);
+    p += ld;
+    ++k;
+  }
+  uint32_t y = (uint32_t)x;
+  for (; k + 1 < n; ++k) {
+    const uint32_t d = (uint32_t)div[k].d;   // widths are below 2^31
+    uint32_t q = __umulhi(y, div[k].r32), m = y - q * d;
+    if (m >= d) { ++q; m -= d; }
+    *p = (int32_t)m + lo[k];
+    p += ld;
+    y = q;
+  }
+  if (n > 0) *p = (int32_t)y + lo[k];   // (the last digit is below its width, so it fits)
 }
 
 // Exponents of the polynomial part of an output code (the inverse of the
@@ -344,18 +404,14 @@ __device__ __forceinline__ int64_t divmod_nn(int64_t x, int64_t d, int64_t* r) {
 __device__ __forceinline__ void decode_poly_part(const Prod& P, int64_t pc, int32_t* __restrict__ exps,
                                                  int64_t ld, int64_t q) {
   if (!P.graded) {
-    for (int k = 0; k < P.np; ++k) {
-      int64_t d = pc;
-      if (k + 1 < P.np) pc = divmod_nn(pc, P.w[k], &d);
-      exps[(int64_t)k * ld + q] = (int32_t)(d + P.omin[k]);
-    }
+    decode_digits(P.div, P.omin, P.np, pc, exps + q, ld);
     return;
   }
   int64_t deg_rest = 0;
   for (int k = 0; k < P.np; ++k) {
     if (k == P.gvar) continue;
     int64_t d;
-    pc = divmod_nn(pc, P.w[k], &d);
+    pc = divmod(pc, P.div[k], &d);
     const int64_t e = d + P.omin[k];
     if ((P.gmask >> k) & 1u) deg_rest += e;
     exps[(int64_t)k * ld + q] = (int32_t)e;
@@ -372,17 +428,11 @@ __device__ __forceinline__ void decode_pseries_term(const Prod& P, int64_t key, 
   const int64_t per_kind = P.T2 * P.Wp;
   const int64_t kd = key >= per_kind ? 1 : 0;   // keys lie below 2 * per_kind
   int64_t pc;
-  const int64_t T = divmod_nn(key - kd * per_kind, P.Wp, &pc);
+  const int64_t T = divmod(key - kd * per_kind, P.divWp, &pc);
   if (kind) kind[q] = (uint8_t)kd;
   if (exps) decode_poly_part(P, pc, exps, ld, q);
-  if (trig) {
-    int64_t u = T + (P.T2 - 1);   // T2 - 1 = sum_k c_k R_k
-    for (int k = 0; k < P.nt; ++k) {
-      int64_t d = u;
-      if (k + 1 < P.nt) u = divmod_nn(u, P.w[P.np + k], &d);
-      trig[(int64_t)k * ld + q] = (int32_t)(d + P.omin[P.np + k]);
-    }
-  }
+  // T2 - 1 = sum_k c_k R_k
+  if (trig) decode_digits(P.div + P.np, P.omin + P.np, P.nt, T + (P.T2 - 1), trig + q, ld);
 }
 
 // int64 accumulate into shared memory as two 32-bit words (the low word at
@@ -521,20 +571,40 @@ cudaError_t launch_hash_insert(Prod* dprods, const int32_t* dhash_prods, const i
                                int nhash, bool poly, bool pseries, bool trunc, int grid, cudaStream_t s);
 // Windowed accumulation: lists, bucket indexes, histogram and cuts of every
 // listed product (drprefix: nwp + 1 offsets of runs; ddone: a zeroed counter;
-// merging: positions in the list of the `merge` products with Win::merge),
-// then the windows of the products of one kind (max_windows: at most that many)
-// and the copy that puts the products together.  dbefore, dscan: max_windows
-// int64 and a scan's scratch; dbase: where the terms start (null: 0); *dtotal:
-// where they end.
+// merging: positions in the list of the `merge` products with Win::merge).
 cudaError_t launch_win_plan(const Prod* dprods, const int32_t* dwprods, int nwp, bool poisson,
                             const int* merging, int merge,
                             int64_t max_terms, int64_t max_samples, int64_t max_bins, int64_t* drprefix,
                             int64_t slots, int64_t ctas, unsigned int* ddone, cudaStream_t s);
-cudaError_t launch_window(Prod* dprods, const int32_t* dwprods, const int64_t* drprefix, int nwp, int kind,
-                          int64_t max_windows, int64_t* dticket, const WinOut& out, int64_t* dbefore, int64_t* dscan,
-                          const int64_t* dbase, int64_t* dtotal, int64_t cap, uint64_t* okey, uint64_t* oval,
-                          unsigned char* staging, int stage_max, int sms, cudaStream_t s, int* launches);
+// The windows of the listed products of one kind.
+struct WinLaunch {
+  const int32_t* prods = nullptr;     // [nwp] (device)
+  const int64_t* rprefix = nullptr;   // [nwp + 1]
+  int nwp = 0, kind = 0;
+  int64_t max_windows = 0;
+  WinOut out{};
+  int64_t* before = nullptr;          // [max_windows] and the scratch of its scan
+  int64_t* scan = nullptr;
+};
+inline bool win_scanned(const WinLaunch& L) { return L.max_windows > 4096; }
+cudaError_t launch_window(Prod* dprods, const WinLaunch& L, int64_t* dticket, unsigned char* staging, int stage_max,
+                          int sms, cudaStream_t s, int* launches);
 size_t win_staging(int stage_max, int sms);   // bytes of launch_window's staging for the largest Win::stage
+// ... and then the terms together in (okey, oval) (dbase: where they start,
+// null: 0; *dtotal: where they end), or, for a single product, decoded into the
+// caller's device arrays (row stride cap; nothing is written if they are short).
+struct SeriesOut {
+  int32_t* exps;
+  int32_t* trig;
+  uint8_t* kind;
+  int64_t* codes;
+  uint64_t* coef;
+  int64_t cap;
+};
+cudaError_t launch_win_copy(Prod* dprods, const WinLaunch& L, const int64_t* dbase, int64_t* dtotal, int64_t cap,
+                            uint64_t* okey, uint64_t* oval, int sms, cudaStream_t s);
+cudaError_t launch_win_decode(Prod* dprods, const WinLaunch& L, bool series, const SeriesOut& out, int sms,
+                              cudaStream_t s);
 // Compaction: up to this many chunks one pass (each chunk read once, one
 // launch); above it two passes, whose counting pass keeps more loads in
 // flight.

@@ -199,6 +199,8 @@ void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_
     if (kr > lim) { pl.st = KR_ERR_OVERFLOW; return; }
     P.krange = (int64_t)kr;
   }
+  for (int k = 0; k < P.np + P.nt; ++k) P.div[k] = make_divisor(P.w[k]);
+  P.divWp = make_divisor(P.Wp);
   // ---- truncation by harmonic order (Sec. 3), Poisson series: each emitted
   // term is tested in the kernels against the packed multipliers
   if (o.trunc_harmonic) {

@@ -7,13 +7,13 @@
 // work, one CTA forms every pair of a window, accumulates it in a small table
 // in shared memory and orders the window's terms there.  Nothing is cleared,
 // compacted or ordered in device memory.  A window's terms go to the next free
-// stretch of a raw array (no CTA waits for another), and one copy puts the
-// stretches together in key order.
+// stretch of a raw array (no CTA waits for another), and one pass puts the
+// stretches together in key order: the decode of a single product, or a copy.
 //
 // Measured on GB300 (whole calls): 6188 x 6188 terms of the weighted sparse
-// structure 1.90 -> 1.16 ms, 2311 x 1507 random float64 terms over 2.8e11 keys
-// 12.7 -> 0.53 ms (its ordering alone took 11.9), a Poisson product of 5003 x
-// 3989 terms (37 M output terms) 6.5 -> 2.3 ms, 20000 x 20000 (597 M terms) 64.5
+// structure 1.90 -> 1.12 ms, 2311 x 1507 random float64 terms over 2.8e11 keys
+// 12.7 -> 0.45 ms (its ordering alone took 11.9), a Poisson product of 5003 x
+// 3989 terms (37 M output terms) 6.6 -> 2.06 ms, 20000 x 20000 (597 M terms) 64.5
 // -> 45 ms.  The window kernel is bound by instruction issue (60% of the issue
 // slots; 2 CTAs of 512 threads per SM, 110 KB of shared memory each): forming,
 // adding and ordering a pair takes about 20 warp instructions, and the walk over
@@ -1357,31 +1357,32 @@ __global__ void __launch_bounds__(WT, 2) k_window(Prod* __restrict__ prods, cons
 
 // Puts the products together: the terms of run t (windows in product and key
 // order) go from their stretches to the position that the counts of the runs
-// before it give.  base: where the first run's terms go (null: 0); *total: the
-// position after the last run's.  before: the scanned counts, or null (few
-// windows): each CTA adds them up.
-__global__ void __launch_bounds__(256) k_win_copy(Prod* __restrict__ prods, const int32_t* __restrict__ wprods,
-                                                  const int64_t* __restrict__ rprefix, int nwp, const WinOut O,
-                                                  const int64_t* __restrict__ before,
-                                                  const int64_t* __restrict__ base_ptr, int64_t* __restrict__ total,
-                                                  int64_t cap, uint64_t* __restrict__ okey,
-                                                  uint64_t* __restrict__ oval) {
+// before it give.  Terms: what becomes of a term at its position.  base: where
+// the first run's terms go (null: 0); *total: the position after the last
+// run's (null: not wanted).  before: the scanned counts, or null (few windows):
+// each CTA adds them up.  The CTAs of a column of the grid share its runs'
+// stretches: two of them, since runs differ in length (1 to 8 a column are within 2 %).
+constexpr int WIN_PUT_TERMS = 4;   // terms of a thread at once, 256 apart: loads in flight
+template <typename Terms>
+__device__ __forceinline__ void win_put(Prod* prods, const int32_t* wprods, const int64_t* rprefix, int nwp,
+                                        const WinOut& O, const int64_t* before, const int64_t* base_ptr,
+                                        int64_t* total, Terms terms) {
   __shared__ int64_t ws[8];
   const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t nwin = rprefix[nwp];
+  const int64_t nrun = rprefix[nwp];
   const int64_t base = base_ptr ? *base_ptr : 0;
-  for (int64_t t = blockIdx.x; t <= nwin; t += gridDim.x) {
-    const int64_t n = t < nwin ? O.count[t] : 0;
+  for (int64_t t = blockIdx.x; t <= nrun; t += gridDim.x) {
+    const int64_t n = t < nrun ? O.count[t] : 0;
     int lo = 0, hi = nwp - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
       if (rprefix[mid] <= t) lo = mid; else hi = mid - 1;
     }
-    const bool first = t < nwin && rprefix[lo] == t;   // of product lo
-    if (n == 0 && !first && t < nwin) continue;   // uniform
+    const bool first = t < nrun && rprefix[lo] == t;   // of product lo
+    if (n == 0 && !first && t < nrun) continue;   // uniform
     int64_t pos;
     if (before) {
-      pos = t < nwin ? before[t] : before[nwin - 1] + O.count[nwin - 1];
+      pos = t < nrun ? before[t] : before[nrun - 1] + O.count[nrun - 1];
     } else {
       int64_t s = 0;
       for (int64_t x = tid; x < t; x += 256) s += O.count[x];
@@ -1394,34 +1395,133 @@ __global__ void __launch_bounds__(256) k_win_copy(Prod* __restrict__ prods, cons
       __syncthreads();
     }
     pos += base;
-    if (t == nwin) {
-      if (tid == 0) *total = pos;
+    if (t == nrun) {
+      if (tid == 0 && blockIdx.y == 0 && total) *total = pos;
       break;
     }
-    if (first && tid == 0) prods[wprods[lo]].out_start = pos;
+    if (first && tid == 0 && blockIdx.y == 0) prods[wprods[lo]].out_start = pos;
     for (int32_t s = O.head[t] - 1; s >= 0 && n > 0;) {
       const WinSeg g = O.seg[s];
-      const int64_t m = min((int64_t)g.n, min(O.cap - g.pos, cap - pos));
-      constexpr int U = 4;   // loads in flight per thread and array
-      for (int64_t i0 = tid; i0 < m; i0 += 256 * U) {
+      const int64_t m = min((int64_t)g.n, O.cap - g.pos);
+      constexpr int U = WIN_PUT_TERMS;
+      for (int64_t i0 = tid + 256 * U * (int64_t)blockIdx.y; i0 < m; i0 += 256 * U * (int64_t)gridDim.y) {
+        const int cnt = (int)min((int64_t)U, (m - i0 + 255) >> 8);
         uint64_t k[U], v[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (i0 + 256 * u < m) {
+        for (int u = 0; u < U; ++u) {
+          k[u] = v[u] = 0;
+          if (u < cnt) {
             k[u] = __ldcs(O.key + g.pos + i0 + 256 * u);
             v[u] = __ldcs(O.val + g.pos + i0 + 256 * u);
           }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (i0 + 256 * u < m) {
-            okey[pos + i0 + 256 * u] = k[u];
-            oval[pos + i0 + 256 * u] = v[u];
-          }
+        }
+        terms(pos + i0, cnt, k, v);
       }
       pos += g.n;
       s = g.next;
     }
   }
+}
+
+__global__ void __launch_bounds__(256) k_win_copy(Prod* __restrict__ prods, const int32_t* __restrict__ wprods,
+                                                  const int64_t* __restrict__ rprefix, int nwp, const WinOut O,
+                                                  const int64_t* __restrict__ before,
+                                                  const int64_t* __restrict__ base_ptr, int64_t* __restrict__ total,
+                                                  int64_t cap, uint64_t* __restrict__ okey,
+                                                  uint64_t* __restrict__ oval) {
+  win_put(prods, wprods, rprefix, nwp, O, before, base_ptr, total, [&](int64_t q, int cnt, const uint64_t* key, const uint64_t* val) {
+#pragma unroll
+    for (int u = 0; u < WIN_PUT_TERMS; ++u, q += 256)
+      if (u < cnt && q < cap) {
+        okey[q] = key[u];
+        oval[q] = val[u];
+      }
+  });
+}
+
+// decode_digits of a thread's terms, 256 places apart (cnt of them): a digit's
+// divisor is fetched and its row's address formed once for all of them.  At
+// 37 million Poisson terms of seven digits 252 M warp instructions against 354 M
+// for a term at a time, 0.52 against 0.60 ms.
+__device__ __forceinline__ void decode_digits_put(const Divisor* div, const int32_t* lo, int n, uint64_t* x,
+                                                  int cnt, int32_t* __restrict__ p, int64_t ld) {
+  constexpr int U = WIN_PUT_TERMS;
+  for (int k = 0; k < n; ++k, p += ld) {
+    const int32_t l = lo[k];
+    uint32_t m[U];
+    if (k + 1 < n) {
+      const Divisor v = div[k];
+      uint64_t high = 0;
+#pragma unroll
+      for (int u = 0; u < U; ++u) high |= x[u];
+      if (high >> 32) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          int64_t r;
+          x[u] = (uint64_t)divmod((int64_t)x[u], v, &r);
+          m[u] = (uint32_t)r;
+        }
+      } else {
+        const uint32_t d = (uint32_t)v.d;   // widths are below 2^31
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          uint32_t q = __umulhi((uint32_t)x[u], v.r32);
+          m[u] = (uint32_t)x[u] - q * d;
+          if (m[u] >= d) { ++q; m[u] -= d; }
+          x[u] = q;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u) m[u] = (uint32_t)x[u];   // (below the last width)
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (u < cnt) p[256 * u] = (int32_t)m[u] + l;
+  }
+}
+
+// The same for a single product, its terms decoded straight into the caller's
+// arrays: no copy and no second pass.  Bound by its writes (1.43 GB in columns of
+// 4 bytes, 0.76 GB read: 4.2 TB/s) at 37 million Poisson terms: 0.52 ms, against
+// 0.34 + 0.44 ms for a copy and a decode of it with plain divisions.  Nothing is
+// written when the product does not fit the arrays.
+template <bool SERIES>
+__global__ void __launch_bounds__(256) k_win_decode(Prod* __restrict__ prods, const int32_t* __restrict__ wprods,
+                                                    const int64_t* __restrict__ rprefix, const WinOut O,
+                                                    const int64_t* __restrict__ before, const SeriesOut D) {
+  __shared__ Prod s_prod;
+  const Prod& P = shared_prod(&prods[wprods[0]], &s_prod);
+  if (P.status || P.nout > D.cap) return;   // uniform
+  win_put(prods, wprods, rprefix, 1, O, before, nullptr, nullptr, [&](int64_t q, int cnt, const uint64_t* key, const uint64_t* val) {
+    constexpr int U = WIN_PUT_TERMS;
+    uint64_t pc[U], tc[U];
+    const int64_t per_kind = P.T2 * P.Wp;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t code = (int64_t)key[u] + P.klo;   // keys are relative to the key window
+      if (u < cnt) {
+        if (D.codes) D.codes[q + 256 * u] = code;
+        D.coef[q + 256 * u] = val[u];
+      }
+      pc[u] = (uint64_t)code;
+      if (SERIES) {
+        const int64_t kd = code >= per_kind ? 1 : 0;   // keys lie below 2 * per_kind
+        int64_t r;
+        tc[u] = (uint64_t)(divmod(code - kd * per_kind, P.divWp, &r) + (P.T2 - 1));   // T2 - 1 = sum_k c_k R_k
+        pc[u] = (uint64_t)r;
+        if (u < cnt && D.kind) D.kind[q + 256 * u] = (uint8_t)kd;
+      }
+    }
+    if (D.exps && !P.graded) {
+      decode_digits_put(P.div, P.omin, P.np, pc, cnt, D.exps + q, D.cap);
+    } else if (D.exps) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (u < cnt) decode_poly_part(P, (int64_t)pc[u], D.exps, D.cap, q + 256 * u);
+    }
+    if (SERIES && D.trig) decode_digits_put(P.div + P.np, P.omin + P.np, P.nt, tc, cnt, D.trig + q, D.cap);
+  });
 }
 
 // How many pairs share a key, by region of the product's windows: the mean of
@@ -1536,27 +1636,42 @@ size_t win_staging(int stage_max, int sms) {
          std::max(win_staging_bytes<uint32_t, WIN_SLOTS_32>(), win_staging_bytes<uint64_t, WIN_SLOTS_64>());
 }
 
-cudaError_t launch_window(Prod* dprods, const int32_t* dwprods, const int64_t* drprefix, int nwp, int kind,
-                          int64_t max_windows, int64_t* dticket, const WinOut& out, int64_t* dbefore, int64_t* dscan,
-                          const int64_t* dbase, int64_t* dtotal, int64_t cap, uint64_t* okey, uint64_t* oval,
-                          unsigned char* staging, int stage_max, int sms, cudaStream_t s, int* launches) {
-  if (nwp <= 0) return cudaSuccess;
-  cudaError_t e = kind == WIN_32 ? launch_window_t<uint32_t, WIN_SLOTS_32>(dprods, dwprods, drprefix, nwp, dticket, out,
-                                                                           staging, stage_max, sms, s)
-                                 : launch_window_t<uint64_t, WIN_SLOTS_64>(dprods, dwprods, drprefix, nwp, dticket, out,
-                                                                           staging, stage_max, sms, s);
+cudaError_t launch_window(Prod* dprods, const WinLaunch& L, int64_t* dticket, unsigned char* staging, int stage_max,
+                          int sms, cudaStream_t s, int* launches) {
+  if (L.nwp <= 0) return cudaSuccess;
+  cudaError_t e =
+      L.kind == WIN_32
+          ? launch_window_t<uint32_t, WIN_SLOTS_32>(dprods, L.prods, L.rprefix, L.nwp, dticket, L.out, staging, stage_max,
+                                                    sms, s)
+          : launch_window_t<uint64_t, WIN_SLOTS_64>(dprods, L.prods, L.rprefix, L.nwp, dticket, L.out, staging, stage_max,
+                                                    sms, s);
   if (e != cudaSuccess) return e;
-  *launches += 2;
-  const bool scanned = max_windows > 4096;
-  if (scanned) {
-    e = cudaMemcpyAsync(dbefore, out.count, sizeof(int64_t) * (size_t)max_windows, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = launch_scan_exclusive(dbefore, max_windows, nullptr, dscan, s);
-    if (e != cudaSuccess) return e;
+  *launches += 1;
+  if (win_scanned(L)) {
+    e = cudaMemcpyAsync(L.before, L.out.count, sizeof(int64_t) * (size_t)L.max_windows, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = launch_scan_exclusive(L.before, L.max_windows, nullptr, L.scan, s);
     *launches += 1;
   }
-  const int64_t grid = max_windows + 1 < 8 * sms ? max_windows + 1 : 8 * sms;
-  k_win_copy<<<(unsigned)grid, 256, 0, s>>>(dprods, dwprods, drprefix, nwp, out, scanned ? dbefore : nullptr, dbase,
-                                           dtotal, cap, okey, oval);
+  return e;
+}
+
+constexpr int WIN_PUT_PARTS = 2;
+static dim3 put_grid(const WinLaunch& L, int sms) {
+  return dim3((unsigned)std::min<int64_t>(L.max_windows + 1, 8 * (int64_t)sms), WIN_PUT_PARTS);
+}
+
+cudaError_t launch_win_copy(Prod* dprods, const WinLaunch& L, const int64_t* dbase, int64_t* dtotal, int64_t cap,
+                            uint64_t* okey, uint64_t* oval, int sms, cudaStream_t s) {
+  if (L.nwp <= 0) return cudaSuccess;
+  k_win_copy<<<put_grid(L, sms), 256, 0, s>>>(dprods, L.prods, L.rprefix, L.nwp, L.out,
+                                              win_scanned(L) ? L.before : nullptr, dbase, dtotal, cap, okey, oval);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_win_decode(Prod* dprods, const WinLaunch& L, bool series, const SeriesOut& out, int sms,
+                              cudaStream_t s) {
+  auto* fn = series ? k_win_decode<true> : k_win_decode<false>;
+  fn<<<put_grid(L, sms), 256, 0, s>>>(dprods, L.prods, L.rprefix, L.out, win_scanned(L) ? L.before : nullptr, out);
   return cudaGetLastError();
 }
 

@@ -170,3 +170,46 @@ def test_large_series_equal_the_table(kron):
     b = [to_np(x) for x in pseries(kron, f, g, table_slots=1 << 26)[:4]]
     for x, y in zip(a, b):
         assert np.array_equal(x, y)
+
+
+BOXES = {   # widths: least significant first
+    "ones": [1, 1, 1],
+    "one_inside": [7, 1, 5],
+    "powers_of_two": [1 << 16, 2, 1 << 15, 1 << 16, 1 << 15],           # codes up to 2^63 - 1 (less one value of the last)
+    "whole_int": [(1 << 31) - 1],
+    "whole_ints": [(1 << 31) - 1, (1 << 31) - 1, 2],
+    "narrow_wide": [3, (1 << 31) - 1, (1 << 30) - 1],
+    "at_32_bits": [65537, 65535, 3],
+    "many": [2, 3, 5, 7, 11, 13, 17, 19],
+}
+
+
+@pytest.mark.parametrize("box", sorted(BOXES))
+def test_codes_to_digits(kron, box):
+    """Division by the reciprocal: the ends of each digit, codes either side of
+    2^32, the last code of the box.  Whole numbers: every digit is exact."""
+    w = BOXES[box]
+    if box == "powers_of_two":
+        w = w[:-1] + [(1 << 15) - 1]
+    lo = [-(x // 2) for x in w]
+    hi = [a + x - 1 for a, x in zip(lo, w)]
+    rng = np.random.default_rng(71)
+    W = 1
+    codes = {0}
+    for x in w:
+        codes |= {W - 1, W, W * (x - 1), W * x - 1}
+        W *= x
+    assert W < 1 << 63
+    codes |= {W - 1, (1 << 32) - 1, 1 << 32, (1 << 32) + 1} | {int(c) for c in rng.integers(0, W, 500)}
+    codes = sorted(c for c in codes if c < W)
+    want = np.zeros((len(w), len(codes)), np.int32)
+    for i, c in enumerate(codes):
+        for k, x in enumerate(w):
+            want[k, i] = c % x + lo[k]
+            c //= x
+    assert np.array_equal(to_np(kron.kron_decode(dev(np.array(codes, np.int64)), lo, hi)), want)
+    assert np.array_equal(to_np(kron.kron_encode(dev(want), lo, hi)), np.array(codes, np.int64))
+    # and as the digits of a product: one term by every other, the box moved
+    one = Poly(np.zeros((len(w), 1), np.int32), np.array([3], np.int64))
+    ex, cf, _, _ = poly(kron, one, Poly(want, np.arange(1, len(codes) + 1, dtype=np.int64)))
+    assert np.array_equal(to_np(ex), want) and np.array_equal(to_np(cf), 3 * np.arange(1, len(codes) + 1))
