@@ -677,7 +677,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
   std::vector<OpRef> all, bm, bt;
   // large operands with key ranges of at most CL_MAX_BITS, in a call with
   // few of them: the cluster front end (encode, rank and gather by CL_CTAS
-  // CTAs each); the rest: one CTA each (bitmap or bitonic) or the radix sort
+  // CTAs each); the rest: one CTA (bitmap) or a cluster (bitonic) each, or the radix sort
   std::vector<OpRef> cl;
   int ncand = 0;
   int64_t cl_range = 0;
@@ -775,7 +775,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       const Prod& P = plans[live_ids[r.prod]].p;
       mx = std::max(mx, ((r.which ? P.g : P.f).key_range + 1023) / 1024);
     }
-    ck(ctx, launch_sort_small(A.lprods, d_bm, (int)bm.size(), SORT_BITMAP, (size_t)mx * 36 * 4 + 64, s),
+    ck(ctx, launch_sort_bitmap(A.lprods, d_bm, (int)bm.size(), (size_t)mx * 36 * 4 + 64, s),
        "bitmap sort");
     ctx->launches += 1;
   }
@@ -785,8 +785,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       const Prod& P = plans[live_ids[r.prod]].p;
       mx = std::max(mx, (r.which ? P.g : P.f).n);
     }
-    ck(ctx, launch_sort_small(A.lprods, d_bt, (int)bt.size(), SORT_BITONIC, (size_t)mx * 8, s),
-       "bitonic sort");
+    ck(ctx, launch_sort_bitonic(A.lprods, d_bt, (int)bt.size(), mx, s), "bitonic sort");
     ctx->launches += 1;
   }
   for (int q = 0; q < nlive; ++q) {

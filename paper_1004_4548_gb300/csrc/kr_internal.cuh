@@ -504,8 +504,8 @@ size_t range_scan_scratch_bytes(int nops, int64_t max_n);
 cudaError_t launch_range_scan(const Prod* dprods, const OpRef* dops, int nops, int64_t max_n, void* scratch,
                               unsigned int* ddone, int32_t* dranges, cudaStream_t s);
 cudaError_t launch_encode(Prod* dprods, const OpRef* dops, int nops, cudaStream_t s);
-cudaError_t launch_sort_small(Prod* dprods, const OpRef* dops, int nops, int method,
-                              size_t smem, cudaStream_t s);
+cudaError_t launch_sort_bitmap(Prod* dprods, const OpRef* dops, int nops, size_t smem, cudaStream_t s);
+cudaError_t launch_sort_bitonic(Prod* dprods, const OpRef* dops, int nops, int64_t max_n, cudaStream_t s);
 cudaError_t launch_gather(Prod* dprods, const OpRef* dops, int nops, cudaStream_t s);
 // SORT_CLUSTER operands: encode, bitmap rank and gather (and the g bucket
 // index of a dense product) in one launch of one cluster per operand

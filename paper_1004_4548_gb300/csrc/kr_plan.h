@@ -22,7 +22,7 @@ constexpr double DENSE_KAPPA = 4.0;
 constexpr int64_t DENSE_POISSON_MAX_BYTES = int64_t(48) << 30;
 constexpr double DENSE_POISSON_KAPPA = 16.0;
 constexpr int64_t BITMAP_MAX_BITS = 1600000;   // on-chip bitmap sort (<= 200 KB)
-constexpr int64_t BITONIC_MAX_N = 16384;       // shared-memory bitonic sort (128 KB)
+constexpr int64_t BITONIC_MAX_N = 16384;       // bitonic sort, in the shared memory of a cluster
 constexpr int64_t DEFAULT_S = 8192;            // dense block: 64 KB of shared memory
 constexpr int64_t MAX_S = 27648;               // 216 KB slice + the 10 KB window table
 // compaction chunks: 8192 dense slots (8 B) or 4096 hash slots (16 B), so that

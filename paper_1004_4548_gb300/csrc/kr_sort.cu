@@ -4,15 +4,20 @@
 // intervals of Sec. 4).  Three sorts, chosen per operand by the host:
 //  * bitmap: keys are distinct and their range fits an on-chip bitmap; the
 //    rank of a key is the number of set bits below it (one pass, O(n + range/32));
-//  * bitonic: a shared-memory bitonic network over (key << idx_bits | index)
-//    words for n <= 16384 (all merges ascending, so padding to a power of two
-//    needs no storage);
+//  * bitonic: (key << idx_bits | index) words, n <= 16384: tiles sorted by a
+//    bitonic network in the shared memory of a cluster's CTAs, and ranked
+//    against one another;
 //  * radix: device-wide LSD radix sort of (key, payload) pairs, 8-bit digits,
 //    also used for the hash-path output.
 // Plus a single-CTA exclusive scan used by the compaction and the radix sort.
+#include <cooperative_groups.h>
+
 #include "kr_internal.cuh"
+#include "kr_plan.h"
 
 namespace kr {
+
+namespace cg = cooperative_groups;
 
 // ---------------------------------------------------------------------------
 // block-wide exclusive scan of int64 values held one per thread
@@ -179,58 +184,115 @@ __global__ void __launch_bounds__(1024) k_bitmap_sort(Prod* __restrict__ prods,
 }
 
 // ---------------------------------------------------------------------------
-// bitonic sort of n <= 16384 packed words in shared memory (one CTA per operand)
+// sort of n <= 16384 distinct packed words: the cluster's CTAs sort a tile each
+// in shared memory, and a word's rank is its place in its tile plus the numbers
+// of smaller words in the others, found through distributed shared memory.
+//
+// Bound by the chain of barriers (and of remote loads in the searches), so the
+// tiles are small: 45 to 66 steps of one or two pairs a thread, those within a
+// warp's 64 words without a CTA barrier, then 10 to 12 search steps over all
+// the other tiles at once.  One CTA sorting the whole operand took 78 to 91
+// steps of up to 8 pairs (both operands of 6188 terms: 93 -> 32 us, 2311 and 1507
+// terms: 48 -> 20 us).  Up to BS_MIN terms a cluster has nothing to share.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_bitonic_sort(Prod* __restrict__ prods,
-                                                       const OpRef* __restrict__ ops) {
-  extern __shared__ uint64_t sk[];
-  const OpRef r = ops[blockIdx.x];
+constexpr int BS_THREADS = 512;
+constexpr int BS_CTAS = 8;                         // the portable cluster size
+constexpr int BS_TILE = BITONIC_MAX_N / BS_CTAS;   // words of a tile at most (16 KB)
+constexpr int BS_MIN = 512;                        // words that one CTA sorts alone: a pair or less a thread
+
+template <int CTAS>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(BS_THREADS)
+    k_bitonic_sort(Prod* __restrict__ prods, const OpRef* __restrict__ ops) {
+  __shared__ uint64_t sk[BS_TILE];
+  const int rank = (int)(blockIdx.x % CTAS);
+  const OpRef r = ops[blockIdx.x / CTAS];
   Prod& P = prods[r.prod];
   Operand& O = r.which ? P.g : P.f;
   const int n = (int)O.n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) sk[i] = O.skey[i];
+  const int tile = max((n + CTAS - 1) / CTAS, BS_MIN);
+  const int lo = min(rank * tile, n), m = min(tile, n - lo);
+  for (int i = threadIdx.x; i < m; i += BS_THREADS) sk[i] = O.skey[lo + i];
   __syncthreads();
-  int N = 1;
-  while (N < n) N <<= 1;
-  const int pairs = N >> 1;
-  for (int size = 2; size <= N; size <<= 1) {
-    const int half = size >> 1;
-    // merge two ascending runs: compare i with its mirror in the block of `size`
-    for (int p = threadIdx.x; p < pairs; p += blockDim.x) {
-      const int blk = p / half, off = p - blk * half;
-      const int i = blk * size + off, j = blk * size + size - 1 - off;
-      if (j < n) {
-        uint64_t a = sk[i], b = sk[j];
-        if (a > b) { sk[i] = b; sk[j] = a; }
-      }
+  // all merges ascending: a place at or above m holds no word and is never
+  // compared, so padding to a power of two needs no storage
+  auto order = [&](int i, int j) {
+    if (j < m) {
+      const uint64_t a = sk[i], b = sk[j];
+      if (a > b) { sk[i] = b; sk[j] = a; }
     }
-    __syncthreads();
-    for (int stride = half >> 1; stride > 0; stride >>= 1) {
-      for (int p = threadIdx.x; p < pairs; p += blockDim.x) {
-        const int i = (p / stride) * 2 * stride + (p % stride), j = i + stride;
-        if (j < n) {
-          uint64_t a = sk[i], b = sk[j];
-          if (a > b) { sk[i] = b; sk[j] = a; }
-        }
+  };
+  // 32 pairs in sequence lie in 64 words in sequence where the words of a pair
+  // are that near, and a warp has the same pairs in every such step
+  auto barrier = [](bool own, bool next_own) {
+    if (own && next_own) __syncwarp(); else __syncthreads();
+  };
+  for (int lg = 1; (1 << (lg - 1)) < m; ++lg) {
+    const int size = 1 << lg, half = size >> 1;
+    int pairs = half;
+    while (2 * pairs < m) pairs <<= 1;
+    // merge two ascending runs: compare i with its mirror in the block of `size`
+    for (int p = threadIdx.x; p < pairs; p += BS_THREADS) {
+      const int blk = (p >> (lg - 1)) << lg, off = p & (half - 1);
+      order(blk + off, blk + size - 1 - off);
+    }
+    barrier(size <= 64, true);   // (the step after it spans size / 4, or is the mirror of 4)
+    for (int ls = lg - 2; ls >= 0; --ls) {
+      const int stride = 1 << ls;
+      for (int p = threadIdx.x; p < pairs; p += BS_THREADS) {
+        const int i = ((p >> ls) << (ls + 1)) + (p & (stride - 1));
+        order(i, i + stride);
       }
-      __syncthreads();
+      barrier(stride <= 32, ls > 0 ? stride <= 64 : size <= 32);
     }
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) O.skey[i] = sk[i];
+  __syncthreads();
+  if (CTAS == 1 || n <= tile) {   // (uniform over the cluster: the others have no words)
+    for (int i = threadIdx.x; i < m; i += BS_THREADS) O.skey[lo + i] = sk[i];
+    return;
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();   // every tile is sorted; and every word of O.skey is read before any is written
+  const uint64_t* peer[CTAS];
+  int len[CTAS];
+#pragma unroll
+  for (int c = 0; c < CTAS; ++c) {
+    peer[c] = cl.map_shared_rank(sk, c);
+    len[c] = c == rank ? 0 : max(0, min(tile, n - c * tile));
+  }
+  int top = 1;
+  while (2 * top <= tile) top <<= 1;
+  for (int i = threadIdx.x; i < m; i += BS_THREADS) {
+    const uint64_t x = sk[i];
+    int below[CTAS];
+#pragma unroll
+    for (int c = 0; c < CTAS; ++c) below[c] = 0;
+    for (int step = top; step > 0; step >>= 1) {
+#pragma unroll
+      for (int c = 0; c < CTAS; ++c) {
+        const int t = below[c] + step;
+        if (t <= len[c] && peer[c][t - 1] < x) below[c] = t;
+      }
+    }
+    int at = i;
+#pragma unroll
+    for (int c = 0; c < CTAS; ++c) at += below[c];
+    O.skey[at] = x;
+  }
+  cl.sync();   // no CTA leaves while its tile is searched
 }
 
-cudaError_t launch_sort_small(Prod* dprods, const OpRef* dops, int nops, int method, size_t smem,
-                              cudaStream_t s) {
+cudaError_t launch_sort_bitmap(Prod* dprods, const OpRef* dops, int nops, size_t smem, cudaStream_t s) {
   if (nops <= 0) return cudaSuccess;
-  if (method == SORT_BITMAP) {
-    cudaError_t e = raise_smem_limit((const void*)k_bitmap_sort, (size_t)smem);
-    if (e != cudaSuccess) return e;
-    k_bitmap_sort<<<nops, 1024, smem, s>>>(dprods, dops);
-  } else {
-    cudaError_t e = raise_smem_limit((const void*)k_bitonic_sort, (size_t)smem);
-    if (e != cudaSuccess) return e;
-    k_bitonic_sort<<<nops, 1024, smem, s>>>(dprods, dops);
-  }
+  cudaError_t e = raise_smem_limit((const void*)k_bitmap_sort, (size_t)smem);
+  if (e != cudaSuccess) return e;
+  k_bitmap_sort<<<nops, 1024, smem, s>>>(dprods, dops);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sort_bitonic(Prod* dprods, const OpRef* dops, int nops, int64_t max_n, cudaStream_t s) {
+  if (nops <= 0) return cudaSuccess;
+  if (max_n <= BS_MIN) k_bitonic_sort<1><<<nops, BS_THREADS, 0, s>>>(dprods, dops);
+  else k_bitonic_sort<BS_CTAS><<<(unsigned)nops * BS_CTAS, BS_THREADS, 0, s>>>(dprods, dops);
   return cudaGetLastError();
 }
 

@@ -213,3 +213,23 @@ def test_codes_to_digits(kron, box):
     one = Poly(np.zeros((len(w), 1), np.int32), np.array([3], np.int64))
     ex, cf, _, _ = poly(kron, one, Poly(want, np.arange(1, len(codes) + 1, dtype=np.int64)))
     assert np.array_equal(to_np(ex), want) and np.array_equal(to_np(cf), 3 * np.arange(1, len(codes) + 1))
+
+
+@pytest.mark.parametrize("n", [2, 3, 31, 33, 63, 65, 129, 511, 512, 513, 514, 1025, 4095, 4097, 6188, 9001, 16383, 16384])
+def test_terms_in_any_order(kron, n):
+    """Operand ordering at the edges of its tiles: random and reversed orders,
+    one term by all (int64: exact), and a duplicate across the whole operand."""
+    rng = np.random.default_rng(n)
+    x = np.sort(rng.choice(40 * n + 100, n, replace=False)).astype(np.int32)
+    e = np.stack([x, (x % 7).astype(np.int32) * 1000003])      # ascending in the second variable, then the first
+    coef = np.arange(1, n + 1, dtype=np.int64)
+    one = Poly(np.array([[5], [-3]], np.int32), np.array([-2], np.int64))
+    by_code = np.lexsort((e[0], e[1]))
+    for order in (rng.permutation(n), by_code[::-1]):
+        ex, cf, _, _ = poly(kron, one, Poly(np.ascontiguousarray(e[:, order]), coef[order]))
+        assert np.array_equal(to_np(ex), e[:, by_code] + np.array([[5], [-3]]))
+        assert np.array_equal(to_np(cf), -2 * coef[by_code])
+    e[:, 0] = e[:, -1]
+    with pytest.raises(kron.KronError) as err:
+        poly(kron, one, Poly(np.ascontiguousarray(e), coef))
+    assert err.value.status == kron.KR_ERR_DUP
