@@ -128,9 +128,6 @@ class Clocks:
 # one ncu capture of the kernel on it; valid only for the kernel source it was
 # taken on, identified by the leading hex digits of its SHA-256.
 DENSE_TRAFFIC = {"source": "kr_dense.cu", "source_sha256": "9d91294c0d87e967", "bytes": 2740480}
-# DRAM traffic of the polynomial hash insert kernel on the MP-sparse product,
-# per launch (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture)
-HASH_TRAFFIC = {"source": "kr_hash.cu", "source_sha256": "5724b523f77891fd", "bytes": 590288640 + 641475328}
 
 
 def kernel_traffic(rec):
@@ -416,10 +413,10 @@ def main():
         if sel("hash_cfg3"):
             h3 = time_poly(kron, ctx, *workload_cfg3(), dev, stream, flush, "hash_insert",
                            max(3, args.steps // 2))
-            # 24 B per term-product: an 8 B key probe read, an 8 B coefficient read and write
-            roof3 = hbm_roofline("k_hash_insert_poly", h3["term_products"], h3["kernel_ms"], 24, hbm,
-                                 kernel_traffic(HASH_TRAFFIC))
-            # the ceiling of the same insert routine on random keys, at this product's
+            # the windows accumulate on chip and write 16 B per output term
+            roof3 = hbm_roofline("k_window", h3["term_products"], h3["kernel_ms"],
+                                 16.0 * h3["output_terms"] / h3["term_products"], hbm)
+            # the ceiling of a table in device memory on random keys, at this product's
             # table size (2^24 slots) and key count, and of plain random adds
             ins = kron.kr_probe_table_update_rate(24, h3["output_terms"], h3["term_products"], 0, local, 3)
             add = kron.kr_probe_table_update_rate(24, h3["output_terms"], h3["term_products"], 1, local, 3)
@@ -848,14 +845,15 @@ def time_pseries(kron, ctx, f, g, dev, stream, flush, steps, path=0, hbm_gbs=Non
     tp = f.n * g.n
     ms = statistics.mean(times)
     kms = statistics.mean(kt)
-    form = "hash" if path == 2 else "dense"   # the automatic choice is the dense array here
+    windowed = kernel_name is None   # untruncated: key windows on chip on either path here, 16 B per output term
+    form = "windows" if windowed else "hash" if path == 2 else "dense"
     r = {"value": tp / (ms * 1e-3) / 1e6, "unit": UNIT, "ms_per_step": ms, "term_products": tp,
          "output_terms": int(out[3].shape[0]), "kernel": "hash_insert", "kernel_ms": kms,
          "kernel_rate": tp / (kms * 1e-3) / 1e6, "accumulator": form,
          "stages_ms_last_step": dict(ctx.stages())}
     if hbm_gbs:
-        r["roofline"] = hbm_roofline(kernel_name or "k_hash_insert_pseries", tp, kms, POISSON_BYTES[form],
-                                     hbm_gbs)
+        r["roofline"] = hbm_roofline(kernel_name or "k_window", tp, kms,
+                                     16.0 * int(out[3].shape[0]) / tp if windowed else POISSON_BYTES[form], hbm_gbs)
     return r
 
 

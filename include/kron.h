@@ -129,6 +129,10 @@ typedef struct {
 typedef struct {
   int32_t path;          /* kr_path; AUTO picks by density (Sec. 3.2) */
   int32_t block_slots;   /* dense path: output codes per block (shared-memory slice) */
+  /* The hash path accumulates by windows of the output keys, on chip; setting
+   * probe_limit, max_regrow or table_slots asks for one table in device memory
+   * (as truncation by coefficients or harmonic order does), which load_factor
+   * and unsorted also concern. */
   double load_factor;    /* hash path: target table load factor, (0, 0.9] */
   int32_t probe_limit;   /* hash path: windows probed before TABLE_FULL */
   int32_t unsorted;      /* hash path: 1 = leave the output in table order */
@@ -256,7 +260,8 @@ kr_status kron_decode(kr_ctx* ctx, const int64_t* codes, int64_t n, int32_t nvar
  * the product's box (widths of the output, each operand offset by its own
  * minimum), so a code sum is the product's code.  Dense path (Sec. 3.1): the
  * output code range is split into blocks, each accumulated in on-chip shared
- * memory; hash path (Sec. 3.2): an open-addressing table in device memory.
+ * memory; hash path (Sec. 3.2): open-addressing tables, on chip for one window
+ * of the output codes after another, or one in device memory.
  * Returns KR_ERR_CAPACITY with h->nterms = required when h->capacity is too
  * small: the product is kept in the context and kron_fetch_poly copies it out
  * without recomputing.  Synchronises the stream. */
@@ -265,8 +270,9 @@ kr_status poly_mul(kr_ctx* ctx, const kr_poly* f, const kr_poly* g, kr_poly_out*
 
 /* h = f * g for Poisson series (Eq. 1, Eq. 6 with the factor 1/2).  Dense
  * path (Sec. 3.1): each pair adds into an array indexed by the key of the sum
- * and of the difference term (up to 48 GiB); hash path (Sec. 3.2): both terms
- * go into the open-addressing table.  AUTO picks the dense path when the key
+ * and of the difference term (up to 48 GiB), or into windows of the keys on
+ * chip where few keys of a large array would be hit; hash path (Sec. 3.2): both
+ * terms go into open-addressing tables, as for polynomials.  AUTO picks the dense path when the key
  * range is at most sixteen times the number of updates.
  * Polynomial exponents are coded in the product's box; trig multipliers in the
  * symmetric box |t_k| <= R_k = max|f_k| + max|g_k|, so that sums and
