@@ -635,7 +635,10 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
         O.cap = terms;
         O.key = b.take<uint64_t>(terms);
         O.val = b.take<uint64_t>(terms);
-        O.nseg = nw ? 16 * nw + 4096 : 0;
+        // pieces: a window whose keys cluster is halved down to each cluster, up to
+        // about 20 (32-bit offsets) or 36 times (64-bit), and a cluster that fills
+        // a table takes more than half the pairs of a window
+        O.nseg = nw ? (k ? 40 : 16) * nw + 4096 : 0;
         O.seg = b.take<WinSeg>(O.nseg);
       }
       Z.wstage = b.take<unsigned char>((int64_t)win_staging(win_stage, ctx->num_sms));
