@@ -912,7 +912,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     mark(ctx, s, "zero_accumulators");
     if (!dense_ids.empty()) {
       bool clipped = false;
-      for (int p : dense_ids) clipped |= plans[p].p.clip != 0;
+      for (int p : dense_ids) clipped |= plans[p].p.work_target == 0;
       ck(ctx, launch_dense_plan(A.lprods, A.dense_ids, A.block_begin, (int)dense_ids.size(),
                                 nblocks_total, clipped, A.tasks, dense_tasks_total, Z.counters, s),
          "dense plan");

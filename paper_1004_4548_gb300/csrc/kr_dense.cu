@@ -90,8 +90,9 @@ __device__ __forceinline__ bool block_work(const Prod* prods, const int32_t* den
   return true;
 }
 
-// Work of every clipped product (truncated, or a key window), which its tasks
-// are sized by (of an unclipped one the number of pairs is known).
+// Work of every large clipped product (truncated, or a key window), which its
+// tasks are sized by (of an unclipped one the number of pairs is known, and a
+// small one's tasks have the least size).
 __global__ void __launch_bounds__(PLAN_THREADS) k_dense_work(Prod* __restrict__ prods,
                                                              const int32_t* __restrict__ dense_prods,
                                                              const int64_t* __restrict__ block_begin, int ndense) {

@@ -535,7 +535,7 @@ __host__ __device__ inline int64_t dense_work_target(double pairs, double ctas, 
   const double tgt = pairs / (ctas * per_cta), least = 0.5 * (double)S;
   return (int64_t)(tgt > least ? tgt : least) + 1;
 }
-// clipped: some product is truncated or a key window (its pairs are counted first)
+// clipped: some product is truncated or a key window and large (its pairs are counted first)
 cudaError_t launch_dense_plan(Prod* dprods, const int32_t* ddense_prods,
                               const int64_t* dblock_begin, int ndense, int64_t nblocks_total, bool clipped,
                               DenseTask* dtasks, int64_t task_cap, int64_t* dtask_count,
