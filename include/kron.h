@@ -446,6 +446,17 @@ double kr_probe_alu_rate(int32_t device, int32_t kind, int32_t reps);
  * device stays usable.  Allocates and frees 128 bytes; synchronises the device. */
 kr_status kr_selftest_bounded_wait(int32_t device);
 
+/* Self-test of what the library does when a windowed product (the hash path's
+ * key windows) meets a limit: lowers a limit of one context, so that small
+ * products meet it.  value <= 0 restores the limit.  No kernel runs; the
+ * context's results stay right whatever the limits.
+ * KR_LIMIT_WINDOW_BYTES: output room above which the distinct terms are
+ *   estimated first, in bytes
+ * KR_LIMIT_WINDOW_ROOM: output room per estimated term (below 1 the estimate is
+ *   always short) */
+enum { KR_LIMIT_WINDOW_BYTES = 0, KR_LIMIT_WINDOW_ROOM = 1 };
+kr_status kr_selftest_limit(kr_ctx* ctx, int32_t which, double value);
+
 #ifdef __cplusplus
 }
 #endif

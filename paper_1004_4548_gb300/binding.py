@@ -80,6 +80,7 @@ SIGNATURES = {
     "kr_probe_smem_atomic_rate": (ctypes.c_double, [_i32, _i32, _i32]),
     "kr_probe_smem_accumulate_rate": (ctypes.c_double, [_i32, _i32]),
     "kr_selftest_bounded_wait": (ctypes.c_int, [_i32]),
+    "kr_selftest_limit": (ctypes.c_int, [_vp, _i32, ctypes.c_double]),
     "kr_probe_table_update_rate": (ctypes.c_double, [_i32, _i32, _i64, _i64, _i32, _i32]),
     "kr_probe_alu_rate": (ctypes.c_double, [_i32, _i32, _i32]),
     "kron_dense_product_static": (ctypes.c_int, [_vp, _vp, _i64, _vp, _vp, _i64, ctypes.c_int, _i64,
@@ -355,6 +356,14 @@ def kr_selftest_bounded_wait(device: int = 0) -> int:
     """Status of the bounded-wait self-test: KR_ERR_TIMEOUT when a wait on a
     predecessor that never publishes gave up and was reported."""
     return int(load().kr_selftest_bounded_wait(device))
+
+
+KR_LIMIT_WINDOW_BYTES, KR_LIMIT_WINDOW_ROOM = 0, 1
+
+
+def kr_selftest_limit(ctx: Context, which: int, value: float = 0.0):
+    """Lowers (value > 0) or restores a limit of windowed products in one context."""
+    _check(ctx.L, ctx.h, ctx.L.kr_selftest_limit(ctx.h, which, value), "kr_selftest_limit")
 
 
 def kr_probe_smem_accumulate_rate(device: int = 0, reps: int = 5) -> float:

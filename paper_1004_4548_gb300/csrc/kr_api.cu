@@ -77,6 +77,9 @@ struct kr_ctx {
   uint64_t* raw_key = nullptr;
   uint64_t* raw_val = nullptr;
   int64_t* raw_total = nullptr;
+  // limits of windowed products, lowered by the self-tests only
+  double win_bound = WIN_BOUND_BYTES;   // output room above which the terms are estimated first
+  double win_room = WIN_ROOM;           // room per estimated term
   // stage timing (CUDA events on the call's stream) and launch counting
   bool profile = false;
   std::vector<cudaEvent_t> ev;
@@ -413,7 +416,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       win_bound += 32.0 * std::min((plans[p].p.nt > 0 ? 2.0 : 1.0) * (double)plans[p].p.f.n * (double)plans[p].p.g.n,
                                    (double)plans[p].p.kspan);
   }
-  const bool win_estimate = win_bound > WIN_BOUND_BYTES;
+  const bool win_estimate = win_bound > ctx->win_bound;
   for (int p = 0; p < nprod; ++p) {
     if (plans[p].st != KR_OK) continue;
     if (plans[p].empty) {   // truncated to nothing: a zero product
@@ -595,7 +598,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     out_total = 0, nchunks_total = 0, bins_total = 0, scan_b2 = 0, max_hash_out = 0;
     for (int p : hll_ids) {
       Plan& pl = plans[p];
-      finish_hash_sizes(ins[p].opts, &pl);
+      finish_hash_sizes(ins[p].opts, ctx->win_room, &pl);
       if (pl.p.win.kind) continue;   // its terms come out ordered
       max_hash_out = std::max(max_hash_out, pl.out_cap);
       const int64_t nb = order_bins(pl.p.kspan);
@@ -739,7 +742,10 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     auto put = [&](const void* dst, const void* src, size_t bytes) {
       if (bytes) memcpy(st + ((const char*)dst - dbase), src, bytes);
     };
-    for (int q = 0; q < nlive; ++q) hl[q] = plans[live_ids[q]].p;
+    for (int q = 0; q < nlive; ++q) {
+      hl[q] = plans[live_ids[q]].p;
+      hl[q].nout = 0;   // (a replay's plans hold the prepared run's counts, and windows add to theirs)
+    }
     put(A.lprods, hl, sizeof(Prod) * nlive);
     put(A.oplists, lists.data(), sizeof(OpRef) * lists.size());
     put(A.dense_ids, h_dense_local.data(), 4 * h_dense_local.size());
@@ -899,7 +905,10 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     Bump hb2 = (ctx->replay || deferred) ? hb : Bump(ctx->pinned);
     Prod* hl2 = hb2.take<Prod>(nlive);
     if (!deferred) {   // a deferred product's phase B2 plan went up with phase B1's
-      for (int q = 0; q < nlive; ++q) hl2[q] = plans[live_ids[q]].p;
+      for (int q = 0; q < nlive; ++q) {
+        hl2[q] = plans[live_ids[q]].p;
+        hl2[q].nout = 0;   // (as a repeated phase's plans hold the counts of the attempt before)
+      }
       ck(ctx, cudaMemcpyAsync(A.lprods, hl2, sizeof(Prod) * nlive, cudaMemcpyHostToDevice, s), "upload plan");
       int64_t* st = hb2.take<int64_t>(nlive + 1);
       memcpy(st, h_chunk_begin.data(), 8 * (size_t)(nlive + 1));
@@ -999,11 +1008,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       res[p].err = Z.counters + 3;
       return;
     }
-    if (ctx->replay) {
-      // counts and positions of the prepared run (the replayed compaction
-      // writes the same ones; the caller verifies after the launch)
-      for (int q = 0; q < nlive; ++q) hl2[q] = plans[live_ids[q]].p;
-    } else {
+    if (!ctx->replay) {   // (a replay takes the prepared run's counts: the caller verifies them after the launch)
       ck(ctx, cudaMemcpyAsync(hl2, A.lprods, sizeof(Prod) * nlive, cudaMemcpyDeviceToHost, s), "download");
       int64_t* herr = hb2.take<int64_t>(1);
       ck(ctx, cudaMemcpyAsync(herr, Z.counters + 3, sizeof(int64_t), cudaMemcpyDeviceToHost, s), "download");
@@ -1018,7 +1023,8 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     bool retry = false;
     for (int q = 0; q < nlive; ++q) {
       const int p = live_ids[q];
-      Prod& P = hl2[q];
+      // (a replay's upload is captured: hl2 stays as it was uploaded)
+      const Prod& P = ctx->replay ? plans[p].p : hl2[q];
       plans[p].p.nout = P.nout;
       plans[p].p.out_start = P.out_start;
       if (!ctx->replay && !plans[p].outcap_full && !(P.status & ~ST_OUTCAP) &&
@@ -1468,6 +1474,15 @@ kr_status kr_ctx_stage(const kr_ctx* ctx, int32_t i, const char** name, double* 
   if (name) *name = ctx->stage_name[i];
   if (ms) *ms = ctx->stage_ms[i];
   return KR_OK;
+}
+
+kr_status kr_selftest_limit(kr_ctx* ctx, int32_t which, double value) {
+  if (!ctx) return KR_ERR_INVALID;
+  switch (which) {
+    case KR_LIMIT_WINDOW_BYTES: ctx->win_bound = value > 0.0 ? value : WIN_BOUND_BYTES; return KR_OK;
+    case KR_LIMIT_WINDOW_ROOM: ctx->win_room = value > 0.0 ? value : WIN_ROOM; return KR_OK;
+  }
+  return KR_ERR_INVALID;
 }
 
 int64_t kr_ctx_launch_count(const kr_ctx* ctx) { return ctx ? ctx->launches : 0; }

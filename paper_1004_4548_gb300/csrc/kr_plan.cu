@@ -355,11 +355,11 @@ void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_
   }
 }
 
-void finish_hash_sizes(const kr_opts& o, Plan* pl) {
+void finish_hash_sizes(const kr_opts& o, double win_room, Plan* pl) {
   Prod& P = pl->p;
   if (P.win.kind) {   // no table; the estimate, where there is one, bounds the output room
     const double all = std::min((P.nt > 0 ? 2.0 : 1.0) * (double)P.f.n * (double)P.g.n, (double)P.kspan);
-    pl->out_cap = (int64_t)(P.hll_est > 0.0 && !pl->outcap_full ? std::min(all, P.hll_est * 1.1 + 4096.0) : all);
+    pl->out_cap = (int64_t)(P.hll_est > 0.0 && !pl->outcap_full ? std::min(all, P.hll_est * win_room + 4096.0) : all);
     return;
   }
   const double m = P.nt > 0 ? 2.0 : 1.0;

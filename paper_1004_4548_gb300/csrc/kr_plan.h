@@ -41,6 +41,9 @@ constexpr int64_t WIN_MAX_BINS = 32768;   // histogram bins (132 KB of shared me
 // output room reserved from the bound on the terms up to this many bytes; above
 // it the distinct keys are estimated first
 constexpr double WIN_BOUND_BYTES = 16.0 * 1024 * 1024 * 1024;
+// output room per estimated term: +10% is about six standard errors of the
+// 4096-register HyperLogLog
+constexpr double WIN_ROOM = 1.1;
 constexpr int HASH_TILE_I = 32;
 constexpr int HASH_TILE_J = 1024;
 
@@ -80,6 +83,7 @@ int bits_for(uint64_t range);   // bits needed for values in [0, range)
 
 // Hash path: table size and output capacity from the HyperLogLog estimate of
 // the distinct output keys (or a forced size), capped by the term-product bound.
-void finish_hash_sizes(const kr_opts& o, Plan* pl);
+// win_room: output room per estimated term of a windowed product.
+void finish_hash_sizes(const kr_opts& o, double win_room, Plan* pl);
 
 }  // namespace kr

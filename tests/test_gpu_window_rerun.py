@@ -1,0 +1,86 @@
+"""Windowed products run again: replays of batches that hold no other kind, and
+phase repetitions after a limit was met (lowered limits, so that small products
+meet them)."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.gpu_compare import assert_poly_equal, assert_pseries_close, to_np
+from tests.test_gpu_window import POLY, PSER, dev, poly, pseries
+from workloads import random_poly
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kron():
+    import paper_1004_4548_gb300 as k
+    k.load()
+    return k
+
+
+@pytest.fixture
+def limited(kron):
+    """A context whose limits a test lowers."""
+    ctx = kron.Context()
+    yield lambda which, value: kron.kr_selftest_limit(ctx, which, value) or ctx
+    ctx.close()
+
+
+def up(p):
+    return type(p)(*(dev(x.copy()) for x in vars(p).values()))
+
+
+PREPARED = {
+    "one_32": ([POLY["swapped"]], []),
+    "one_64": ([POLY["offsets_64"]], []),
+    "one_series": ([], [PSER["no_polynomial"]]),
+    "several": ([POLY["swapped"], POLY["offsets_64"], POLY["clustered"]], [PSER["offsets_64"], PSER["cosines"]]),
+}
+
+
+@pytest.mark.parametrize("case", sorted(PREPARED))
+def test_prepared_batch_of_windows_alone(kron, case):
+    import torch
+    polys, series = ([c() for c in cs] for cs in PREPARED[case])
+    pb = kron.PreparedBatch([(up(f), up(g)) for f, g in polys + series], opts={"path": kron.KR_PATH_HASH})
+    want = [r["nterms"] for r in pb.first_results()]
+    for _ in range(3):
+        pb.launch()
+        torch.cuda.synchronize()
+        res = pb.results()
+        assert [r["status"] for r in res] == [0] * len(res) and [r["nterms"] for r in res] == want
+        for r, (f, g) in zip(res, polys):
+            assert_poly_equal(r["exps"], r["coef"], oracle.poly_mul(f, g), case)
+        for r, (f, g) in zip(res[len(polys):], series):
+            assert_pseries_close([r[k] for k in ("exps", "trig", "kind", "coef")], oracle.poisson_mul(f, g, keep_zero=True))
+    pb.close()
+
+
+def test_short_estimate_is_repeated(kron, limited):
+    """The room comes from an estimate that is always short: every product is repeated with full room."""
+    limited(kron.KR_LIMIT_WINDOW_BYTES, 1.0)
+    ctx = limited(kron.KR_LIMIT_WINDOW_ROOM, 0.5)
+    for case in ("offsets_64", "swapped", "one_by_many"):
+        f, g = POLY[case]()
+        r = oracle.poly_mul(f, g)
+        for host in (False, True):
+            ex, cf, _, _ = poly(kron, f, g, ctx=ctx, host_out=host)
+            assert_poly_equal(ex, cf, r, case)
+    f, g = PSER["offsets_64"]()
+    assert_pseries_close(pseries(kron, f, g, ctx=ctx), oracle.poisson_mul(f, g, keep_zero=True))
+    jobs = [POLY["offsets_64"](), POLY["swapped"](), (random_poly(2, 50, 0, 12, 31), random_poly(2, 60, 0, 12, 32))]
+    for n in (2, 3):   # windows alone, and beside a dense product
+        res = kron.kron_mul_batch([(up(f), up(g)) for f, g in jobs[:n]], ctx=ctx)
+        for x, (f, g) in zip(res, jobs):
+            assert x["status"] == 0
+            assert_poly_equal(x["exps"], x["coef"], oracle.poly_mul(f, g))
+
+
+def test_estimated_room(kron, limited):
+    """An estimate that suffices: no repetition, the same terms."""
+    ctx = limited(kron.KR_LIMIT_WINDOW_BYTES, 1.0)
+    f, g = POLY["shared_keys"]()
+    ex, cf, _, _ = poly(kron, f, g, ctx=ctx)
+    assert_poly_equal(ex, cf, oracle.poly_mul(f, g))
+    assert np.array_equal(to_np(cf), to_np(poly(kron, f, g)[1]))
