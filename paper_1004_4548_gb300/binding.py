@@ -320,13 +320,27 @@ def _first_capacity(nf: int, ng: int, per_pair: int, ratio: int, term_bytes: int
     return max(16, n, guess)
 
 
+def _copies_done(t):
+    """Waits for the copies just queued on torch's current stream of t's device: a call's outputs are complete when
+    it returns, for every stream."""
+    if t.is_cuda:
+        _torch().cuda.current_stream(t.device).synchronize()
+
+
 def _trimmed(arrays, n: int, cap: int, guessed: bool):
-    """The first n of cap terms of each array; copies where a guessed capacity would keep over 1 MB of
+    """The first n of cap terms of each array; finished copies where a guessed capacity would keep over 1 MB of
     unused memory alive with them."""
     out = [a if a is None else a[..., :n] for a in arrays]
     if guessed and 2 * n < cap and sum(a.nbytes for a in arrays if a is not None) > 2 << 20:
         out = [a if a is None else a.clone(memory_format=_torch().contiguous_format) for a in out]
+        _copies_done(next(a for a in reversed(out) if a is not None))
     return out
+
+
+def _on_current_stream(sp) -> bool:
+    """Whether a call's stream is torch's current one.  Only then is room guessed and trimmed: the copies run on the
+    current stream, which a caller with a stream of their own should not wait for."""
+    return sp == _stream_ptr(None)
 
 
 # ----------------------------------------------------------------------------
@@ -433,8 +447,10 @@ def poly_mul(f_exps, f_coef, g_exps, g_coef, ctx: Context | None = None, stream=
     f = kr_poly(nv, int(f_exps.shape[1]), pfe, pfc, KR_F64 if is_f64 else KR_I64)
     g = kr_poly(nv, int(g_exps.shape[1]), pge, pgc, KR_F64 if is_f64 else KR_I64)
     o = ctypes.byref(_opts(**opts)) if opts else None   # NULL: the defaults
+    sp = _stream_ptr(stream)
+    guess = capacity is None and (stream is None or _on_current_stream(sp))
     cap = capacity if capacity is not None else \
-        _first_capacity(f.nterms, g.nterms, 1, 1 if opts else 8, 4 * nv + 8)   # options: truncated, a window, ...
+        _first_capacity(f.nterms, g.nterms, 1, 1 if opts or not guess else 8, 4 * nv + 8)   # options: truncated, a window, ...
 
     def outbuf(cap):
         ex = _alloc((nv, cap), np.int32, ctx.device, host_out)
@@ -444,14 +460,13 @@ def poly_mul(f_exps, f_coef, g_exps, g_coef, ctx: Context | None = None, stream=
         return h, ex, cf, cd
 
     h, ex, cf, cd = outbuf(cap)
-    sp = _stream_ptr(stream)
     st = ctx.L.poly_mul(ctx.h, ctypes.byref(f), ctypes.byref(g), ctypes.byref(h), o, sp)
     if st == KR_ERR_CAPACITY:
         h, ex, cf, cd = outbuf(int(h.nterms))
         st = ctx.L.kron_fetch_poly(ctx.h, ctypes.byref(h), sp)
     _check(ctx.L, ctx.h, st, "poly_mul")
     n = int(h.nterms)
-    ex, cf, cd = _trimmed((ex, cf, cd), n, h.capacity, capacity is None)
+    ex, cf, cd = _trimmed((ex, cf, cd), n, h.capacity, guess)
     box = (np.frombuffer(h.omin, np.int32, nv).copy(), np.frombuffer(h.omax, np.int32, nv).copy())
     return ex, cf, cd, box
 
@@ -477,8 +492,11 @@ def poisson_mul(f, g, ctx: Context | None = None, stream=None, capacity: int | N
 
     F, G = desc(f), desc(g)
     o = ctypes.byref(_opts(**opts)) if opts else None   # NULL: the defaults
+    sp = _stream_ptr(stream)
+    guess = capacity is None and (stream is None or _on_current_stream(sp))
     cap = capacity if capacity is not None else \
-        max(2 * (F.nterms + G.nterms), _first_capacity(F.nterms, G.nterms, 2, 1 if opts else 64, 4 * (npoly + ntrig) + 9))
+        max(2 * (F.nterms + G.nterms),
+            _first_capacity(F.nterms, G.nterms, 2, 1 if opts or not guess else 64, 4 * (npoly + ntrig) + 9))
 
     def outbuf(cap):
         ex = _alloc((npoly, cap), np.int32, ctx.device, host_out)
@@ -491,13 +509,12 @@ def poisson_mul(f, g, ctx: Context | None = None, stream=None, capacity: int | N
         return h, ex, tr, kd, cf, cd
 
     h, ex, tr, kd, cf, cd = outbuf(cap)
-    sp = _stream_ptr(stream)
     st = ctx.L.poisson_mul(ctx.h, ctypes.byref(F), ctypes.byref(G), ctypes.byref(h), o, sp)
     if st == KR_ERR_CAPACITY:
         h, ex, tr, kd, cf, cd = outbuf(int(h.nterms))
         st = ctx.L.kron_fetch_pseries(ctx.h, ctypes.byref(h), sp)
     _check(ctx.L, ctx.h, st, "poisson_mul")
-    return tuple(_trimmed((ex, tr, kd, cf, cd), int(h.nterms), h.capacity, capacity is None))
+    return tuple(_trimmed((ex, tr, kd, cf, cd), int(h.nterms), h.capacity, guess))
 
 
 def kron_dense_product_static(fcode, fcoef, gcode, gcoef, W: int, out=None, stream=None):
