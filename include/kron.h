@@ -453,8 +453,10 @@ kr_status kr_selftest_bounded_wait(int32_t device);
  * KR_LIMIT_WINDOW_BYTES: output room above which the distinct terms are
  *   estimated first, in bytes
  * KR_LIMIT_WINDOW_ROOM: output room per estimated term (below 1 the estimate is
- *   always short) */
-enum { KR_LIMIT_WINDOW_BYTES = 0, KR_LIMIT_WINDOW_ROOM = 1 };
+ *   always short)
+ * KR_LIMIT_WINDOW_PIECES: stretches of terms that the windows of a call may put
+ *   down (a product that needs more is done again by the table) */
+enum { KR_LIMIT_WINDOW_BYTES = 0, KR_LIMIT_WINDOW_ROOM = 1, KR_LIMIT_WINDOW_PIECES = 2 };
 kr_status kr_selftest_limit(kr_ctx* ctx, int32_t which, double value);
 
 #ifdef __cplusplus

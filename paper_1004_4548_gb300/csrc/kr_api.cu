@@ -80,6 +80,12 @@ struct kr_ctx {
   // limits of windowed products, lowered by the self-tests only
   double win_bound = WIN_BOUND_BYTES;   // output room above which the terms are estimated first
   double win_room = WIN_ROOM;           // room per estimated term
+  int64_t win_pieces = INT64_MAX;       // stretches of a call
+  // products that their windows could not hold and that run without: by index in
+  // the run's products (found before its end), or the deferred one (found when it
+  // is settled)
+  std::vector<char> win_off;
+  bool win_refused = false;
   // stage timing (CUDA events on the call's stream) and launch counting
   bool profile = false;
   std::vector<cudaEvent_t> ev;
@@ -245,6 +251,7 @@ kr_status status_to_kr(uint32_t st) {
   if (st & ST_INVALID) return KR_ERR_INVALID;
   if (st & ST_RANGE) return KR_ERR_RANGE;
   if (st & ST_DUP) return KR_ERR_DUP;
+  if (st & ST_WINDOW) return KR_ERR_CAPACITY;   // (left to a replay: its plan no longer fits)
   if (st & ST_TABLE_FULL) return KR_ERR_TABLE_FULL;
   if (st & ST_OUTCAP) return KR_ERR_CUDA;
   return KR_OK;
@@ -306,10 +313,12 @@ const T* stage(kr_ctx* ctx, Bump& b, const T* src, int64_t count, cudaStream_t s
 //   B2  (accumulator arena) zero, dense plan + accumulate, hash inserts,
 //       compaction                                      -> sync
 // A product whose table fills up is retried from B2 with a larger table.
-void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
+// False: a product's windows could not hold it (noted in win_off): run again.
+bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
                   std::vector<ProdResult>& res) {
   ctx->attr_memo.clear();
   const int nprod = (int)ins.size();
+  ctx->win_off.resize(nprod, 0);
   res.assign(nprod, ProdResult());
   const int nops = 2 * nprod;
   std::vector<Job> jobs(nprod);
@@ -336,6 +345,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       J.np = in.np;
       J.nt = in.nt;
       J.opts = in.opts;
+      J.no_windows = ctx->win_off[p] != 0;
       J.f.n = in.nf;
       J.g.n = in.ng;
       J.f.e = stage(ctx, b, in.fe, (int64_t)in.np * in.nf, s);
@@ -438,7 +448,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
   std::stable_sort(live_ids.begin(), live_ids.end(),
                    [&](int a, int b) { return plans[a].p.win.kind < plans[b].p.win.kind; });
   const int nlive = (int)live_ids.size();
-  if (nlive == 0) return;
+  if (nlive == 0) return true;
   std::vector<int> local(nprod, -1);
   for (int q = 0; q < nlive; ++q) local[live_ids[q]] = q;
   std::vector<int32_t> h_dense_local, h_hash_local;
@@ -641,7 +651,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
         // pieces: a window whose keys cluster is halved down to each cluster, up to
         // about 20 (32-bit offsets) or 36 times (64-bit), and a cluster that fills
         // a table takes more than half the pairs of a window
-        O.nseg = nw ? (k ? 40 : 16) * nw + 4096 : 0;
+        O.nseg = nw ? std::min(ctx->win_pieces, (k ? 40 : 16) * nw + 4096) : 0;
         O.seg = b.take<WinSeg>(O.nseg);
       }
       Z.wstage = b.take<unsigned char>((int64_t)win_staging(win_stage, ctx->num_sms));
@@ -891,7 +901,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     const int p = live_ids[0];
     res[p].st = status_to_kr(plans[p].p.status);
     res[p].prod = plans[p].p;
-    return;
+    return true;
   }
   // ---------------- phase B2, repeated for products whose table filled up
   std::vector<int> regrows(nprod, 0);
@@ -1006,7 +1016,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       res[p].key = Z.okey;
       res[p].val = Z.oval;
       res[p].err = Z.counters + 3;
-      return;
+      return true;
     }
     if (!ctx->replay) {   // (a replay takes the prepared run's counts: the caller verifies them after the launch)
       ck(ctx, cudaMemcpyAsync(hl2, A.lprods, sizeof(Prod) * nlive, cudaMemcpyDeviceToHost, s), "download");
@@ -1017,16 +1027,21 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       if (*herr) {   // a bounded wait of the compaction gave up: no result is reliable
         ctx->err = "compaction: a wait for a preceding chunk timed out";
         for (int q = 0; q < nlive; ++q) res[live_ids[q]].st = KR_ERR_TIMEOUT;
-        return;
+        return true;
       }
     }
-    bool retry = false;
+    bool retry = false, refused = false;
     for (int q = 0; q < nlive; ++q) {
       const int p = live_ids[q];
       // (a replay's upload is captured: hl2 stays as it was uploaded)
       const Prod& P = ctx->replay ? plans[p].p : hl2[q];
       plans[p].p.nout = P.nout;
       plans[p].p.out_start = P.out_start;
+      if (!ctx->replay && (P.status & ST_WINDOW) && !(P.status & ~(ST_WINDOW | ST_OUTCAP))) {
+        ctx->win_off[p] = 1;
+        refused = true;
+        continue;
+      }
       if (!ctx->replay && !plans[p].outcap_full && !(P.status & ~ST_OUTCAP) &&
           ((P.status & ST_OUTCAP) || (P.win.kind && P.nout > P.out_cap))) {
         // the estimate fell short: rerun with room for a full table
@@ -1055,6 +1070,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       res[p].val = Z.oval + P.out_start;
       if (P.nout > P.out_cap) res[p].st = KR_ERR_CUDA;
     }
+    if (refused) return false;
     if (retry) continue;   // phase B2 again, with the grown tables
     // ---------------- hash outputs: order by key
     mark(ctx, s, "begin");
@@ -1108,7 +1124,7 @@ void run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       }
     }
     mark(ctx, s, "output_sort");
-    return;
+    return true;
   }
 }
 
@@ -1365,6 +1381,42 @@ void keep_result(kr_ctx* ctx, const ProdResult& r, bool poisson) {
   ctx->res_err = r.err;
 }
 
+// A single product through the pipeline and into its outputs (emit), and once
+// more without windows where they could not hold it.  deferred: its count may
+// stay on the device until emit.
+template <typename Emit>
+kr_status run_single(kr_ctx* ctx, const JobIn& in, bool deferred, const DirectOut& direct, cudaStream_t s, Emit emit) {
+  std::vector<ProdResult> res;
+  ctx->win_off.assign(1, 0);
+  for (;;) {
+    ctx->allow_deferred = deferred;
+    ctx->allow_raw = true;
+    ctx->res_raw = false;
+    ctx->direct = direct;
+    ctx->direct_done = false;
+    ctx->win_refused = false;
+    auto reset = [&](bool all) {
+      ctx->allow_deferred = ctx->allow_raw = false;
+      ctx->direct = DirectOut{};
+      if (all) ctx->direct_done = false;
+    };
+    try {
+      const bool done = run_pipeline(ctx, {in}, s, res);
+      reset(!done || res[0].st != KR_OK);
+      if (!done) continue;
+      if (res[0].st != KR_OK) return res[0].st;
+      keep_result(ctx, res[0], in.poisson);
+      const kr_status st = emit();
+      ctx->direct_done = false;
+      if (!ctx->win_refused) return st;
+      ctx->win_off[0] = 1;
+    } catch (...) {
+      reset(true);
+      throw;
+    }
+  }
+}
+
 // After a deferred run: the device-side count, status and wait error of the
 // kept product, read once its decode has been queued.  Synchronises.
 kr_status settle_deferred(kr_ctx* ctx, cudaStream_t s) {
@@ -1383,6 +1435,7 @@ kr_status settle_deferred(kr_ctx* ctx, cudaStream_t s) {
   }
   if (hp_prod->status) {
     ctx->has_result = false;
+    ctx->win_refused = (hp_prod->status & ST_WINDOW) && !(hp_prod->status & ~(ST_WINDOW | ST_OUTCAP));
     return status_to_kr(hp_prod->status);
   }
   ctx->res_n = hp_prod->nout;
@@ -1481,6 +1534,7 @@ kr_status kr_selftest_limit(kr_ctx* ctx, int32_t which, double value) {
   switch (which) {
     case KR_LIMIT_WINDOW_BYTES: ctx->win_bound = value > 0.0 ? value : WIN_BOUND_BYTES; return KR_OK;
     case KR_LIMIT_WINDOW_ROOM: ctx->win_room = value > 0.0 ? value : WIN_ROOM; return KR_OK;
+    case KR_LIMIT_WINDOW_PIECES: ctx->win_pieces = value > 0.0 ? (int64_t)value : INT64_MAX; return KR_OK;
   }
   return KR_ERR_INVALID;
 }
@@ -1631,15 +1685,10 @@ kr_status poly_mul(kr_ctx* ctx, const kr_poly* f, const kr_poly* g, kr_poly_out*
     in.fe = f->exps; in.fc = f->coef; in.nf = f->nterms;
     in.ge = g->exps; in.gc = g->coef; in.ng = g->nterms;
     if (opts) in.opts = *opts;
-    std::vector<ProdResult> res;
     // the term count may stay on the device until the decode (host outputs:
     // until the decode into scratch, whose terms are then copied); with every
     // output in device memory the compaction may decode into it directly
-    ctx->allow_deferred = true;
-    ctx->allow_raw = true;
-    ctx->res_raw = false;
-    ctx->direct = DirectOut{};
-    ctx->direct_done = false;
+    DirectOut direct{};
     if (h->capacity > 0) {
       // device memory, or pinned host memory through its device mapping (the
       // GPU writes the terms across the host link; no copies afterwards)
@@ -1647,31 +1696,14 @@ kr_status poly_mul(kr_ctx* ctx, const kr_poly* f, const kr_poly* g, kr_poly_out*
       void* ex = h->exps ? device_view(h->exps) : nullptr;
       void* cd = h->codes ? device_view(h->codes) : nullptr;
       if (cf && (!h->exps || ex) && (!h->codes || cd)) {
-        ctx->direct.exps = (int32_t*)ex;
-        ctx->direct.codes = (int64_t*)cd;
-        ctx->direct.coef = (uint64_t*)cf;
-        ctx->direct.ld = h->capacity;
-        ctx->direct.cap = h->capacity;
+        direct.exps = (int32_t*)ex;
+        direct.codes = (int64_t*)cd;
+        direct.coef = (uint64_t*)cf;
+        direct.ld = h->capacity;
+        direct.cap = h->capacity;
       }
     }
-    try {
-      run_pipeline(ctx, {in}, s, res);
-    } catch (...) {
-      ctx->allow_deferred = ctx->allow_raw = false;
-      ctx->direct = DirectOut{};
-      ctx->direct_done = false;
-      throw;
-    }
-    ctx->allow_deferred = ctx->allow_raw = false;
-    ctx->direct = DirectOut{};
-    if (res[0].st != KR_OK) {
-      ctx->direct_done = false;
-      return res[0].st;
-    }
-    keep_result(ctx, res[0], false);
-    const kr_status st = emit_poly(ctx, h, s);
-    ctx->direct_done = false;
-    return st;
+    return run_single(ctx, in, true, direct, s, [&]() -> kr_status { return emit_poly(ctx, h, s); });
   });
 }
 
@@ -1706,24 +1738,10 @@ kr_status poisson_mul(kr_ctx* ctx, const kr_pseries* f, const kr_pseries* g, kr_
     in.fe = f->exps; in.ft = f->trig; in.fk = f->kind; in.fc = f->coef; in.nf = f->nterms;
     in.ge = g->exps; in.gt = g->trig; in.gk = g->kind; in.gc = g->coef; in.ng = g->nterms;
     if (opts) in.opts = *opts;
-    std::vector<ProdResult> res;
-    ctx->allow_deferred = is_device_ptr(h->coef) && (!h->exps || is_device_ptr(h->exps)) &&
-                          (!h->trig || is_device_ptr(h->trig)) && (!h->kind || is_device_ptr(h->kind)) &&
-                          (!h->codes || is_device_ptr(h->codes));
-    ctx->allow_raw = true;
-    ctx->res_raw = false;
-    ctx->direct = DirectOut{};
-    ctx->direct_done = false;
-    try {
-      run_pipeline(ctx, {in}, s, res);
-    } catch (...) {
-      ctx->allow_deferred = ctx->allow_raw = false;
-      throw;
-    }
-    ctx->allow_deferred = ctx->allow_raw = false;
-    if (res[0].st != KR_OK) return res[0].st;
-    keep_result(ctx, res[0], true);
-    return emit_pseries(ctx, h, s);
+    const bool all_dev = is_device_ptr(h->coef) && (!h->exps || is_device_ptr(h->exps)) &&
+                         (!h->trig || is_device_ptr(h->trig)) && (!h->kind || is_device_ptr(h->kind)) &&
+                         (!h->codes || is_device_ptr(h->codes));
+    return run_single(ctx, in, all_dev, DirectOut{}, s, [&]() -> kr_status { return emit_pseries(ctx, h, s); });
   });
 }
 
@@ -1752,7 +1770,8 @@ kr_status run_wave(kr_ctx* ctx, const std::vector<JobIn>& ins, const std::vector
                    kr_result* res, cudaStream_t s) {
   std::vector<ProdResult> pr;
   try {
-    run_pipeline(ctx, ins, s, pr);
+    ctx->win_off.assign(ins.size(), 0);
+    while (!run_pipeline(ctx, ins, s, pr)) {}
   } catch (const CudaFail& f) {
     if (f.e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
@@ -1989,7 +2008,7 @@ kr_status kron_batch_prepare(int32_t device, const kr_job* jobs, int32_t njobs, 
     if (b->ins.empty()) return KR_OK;
     // the prepared run
     std::vector<ProdResult> pr;
-    run_pipeline(ictx, b->ins, s, pr);
+    while (!run_pipeline(ictx, b->ins, s, pr)) {}
     std::vector<int> order;
     for (int p = 0; p < (int)b->ins.size(); ++p)
       if (pr[p].dprod) order.push_back(p);
@@ -2155,6 +2174,7 @@ kr_status kron_split_hist(kr_ctx* ctx, const kr_job* job, int32_t nbins, int64_t
     ctx->split_nsamples = nsamples;
     ctx->split_seed = seed;
     ctx->split_hist = hist;
+    ctx->win_off.assign(1, 0);
     std::vector<ProdResult> res;
     try {
       run_pipeline(ctx, {in}, s, res);

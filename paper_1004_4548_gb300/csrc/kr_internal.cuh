@@ -28,6 +28,7 @@ constexpr uint32_t ST_DUP = 2u;         // repeated input key
 constexpr uint32_t ST_INVALID = 4u;     // non-canonical trig input, sine of zero vector
 constexpr uint32_t ST_TABLE_FULL = 8u;  // hash probe limit reached
 constexpr uint32_t ST_OUTCAP = 16u;     // compaction found more terms than reserved
+constexpr uint32_t ST_WINDOW = 32u;     // key windows cannot hold the product: a table has to
 
 // sort method chosen per operand by the host
 constexpr int SORT_BITMAP = 1;   // key range fits an on-chip bitmap

@@ -55,10 +55,11 @@ static void plan_sort(Operand& op, int64_t key_range, int* passes, int64_t* radi
 // Poisson products whose key array would be sparsely hit, unless the caller
 // sized a table or the product is truncated by a criterion that the windows
 // cannot apply by key alone.
-static void plan_window(const kr_opts& o, Plan* out) {
+static void plan_window(const Job& job, Plan* out) {
+  const kr_opts& o = job.opts;
   Prod& P = out->p;
   P.win = Win{};
-  if (P.ctrunc || P.htrunc || (P.graded && P.nt > 0)) return;
+  if (job.no_windows || P.ctrunc || P.htrunc || (P.graded && P.nt > 0)) return;
   if (o.table_slots > 0 || o.probe_limit > 0 || o.max_regrow != 0) return;
   const double m = P.nt > 0 ? 2.0 : 1.0;
   const double updates = m * (double)P.f.n * (double)P.g.n;
@@ -309,7 +310,7 @@ void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_
     P.chunk = COMPACT_CHUNK;
     P.nchunks = ceil_div(P.kspan, P.chunk);
     pl.out_cap = (int64_t)std::min((double)P.kspan, 2.0 * pairs);
-    plan_window(o, &pl);
+    plan_window(job, &pl);
   } else if (P.path == PATH_DENSE) {
     int64_t S = o.block_slots > 0 ? o.block_slots : DEFAULT_S;
     if (S < 256) S = 256;
@@ -351,7 +352,7 @@ void plan_product(const Job& job, const int32_t* rf, const int32_t* rg, int num_
     P.ntasks = ceil_div(nf, HASH_TILE_I) * P.tiles_j;
     P.chunk = COMPACT_CHUNK_HASH;
     // table size, chunks and output capacity follow in finish_hash_sizes
-    plan_window(o, &pl);
+    plan_window(job, &pl);
   }
 }
 

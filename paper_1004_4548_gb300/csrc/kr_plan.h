@@ -54,6 +54,7 @@ struct Job {
   int np = 0, nt = 0;
   Operand f{}, g{};
   kr_opts opts{};
+  bool no_windows = false;   // the hash path's table in device memory (or the key array), whatever the shape
 };
 
 // The result of planning: Prod filled except scratch pointers, plus sizes.

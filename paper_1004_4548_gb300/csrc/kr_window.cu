@@ -1118,19 +1118,20 @@ struct WinRun {
   int32_t last;   // thread 0: the run's newest piece
   int row;        // of the block scans' scratch
 
-  // a stretch of n terms; by every thread
+  // a stretch of n terms (none without terms); by every thread
   __device__ __forceinline__ int64_t place(int n) {
     auto& sh = win_block<KT, SLOTS>().sh;
     if (threadIdx.x == 0) {
       const int64_t pos = (int64_t)atomicAdd(&O.used[0], (unsigned long long)n);
-      const int64_t s = (int64_t)atomicAdd(&O.used[1], 1ull);
+      const int64_t s = n > 0 ? (int64_t)atomicAdd(&O.used[1], 1ull) : -1;
       if (pos + n > O.cap) atomicOr(&P.status, ST_OUTCAP);
-      if (s < O.nseg) {
+      if (s < 0) {
+      } else if (s < O.nseg) {
         O.seg[s] = WinSeg{pos, n, -1};
         if (last < 0) O.head[t] = (int32_t)s + 1; else O.seg[last].next = (int32_t)s;
         last = (int32_t)s;
       } else {
-        atomicOr(&P.status, ST_TABLE_FULL);
+        atomicOr(&P.status, ST_WINDOW);
       }
       sh.excl = pos;
     }

@@ -84,3 +84,34 @@ def test_estimated_room(kron, limited):
     ex, cf, _, _ = poly(kron, f, g, ctx=ctx)
     assert_poly_equal(ex, cf, oracle.poly_mul(f, g))
     assert np.array_equal(to_np(cf), to_np(poly(kron, f, g)[1]))
+
+
+def test_pieces_run_out(kron, limited):
+    """A product whose windows put down more pieces than there is room for goes through the table."""
+    ctx = limited(kron.KR_LIMIT_WINDOW_PIECES, 3)
+
+    def launches(call, c):
+        before = c.launch_count()
+        return call(), c.launch_count() - before
+
+    for case in ("offsets_64", "swapped", "clustered", "clustered_64"):
+        f, g = POLY[case]()
+        r = oracle.poly_mul(f, g)
+        for kw in ({}, {"host_out": True}, {"capacity": 1}, {"capacity": 1, "host_out": True}):
+            (ex, cf, _, _), n = launches(lambda: poly(kron, f, g, ctx=ctx, **kw), ctx)
+            assert_poly_equal(ex, cf, r, f"{case} {kw}")
+            assert n > launches(lambda: poly(kron, f, g, **kw), kron.context())[1]   # the limit was met
+    for case in ("offsets_64", "cosines"):
+        f, g = PSER[case]()
+        r = oracle.poisson_mul(f, g, keep_zero=True)
+        for kw in ({}, {"host_out": True}, {"capacity": 1}):
+            assert_pseries_close(pseries(kron, f, g, ctx=ctx, **kw), r, 1e-12, f"{case} {kw}")
+    dup = random_poly(3, 40, -90, 90, 35)
+    dup.exps[:, 1] = dup.exps[:, 0]
+    jobs = [POLY["offsets_64"](), (random_poly(2, 50, 0, 12, 31), random_poly(2, 60, 0, 12, 32)), POLY["one_by_many"](),
+            (dup, dup), POLY["swapped"]()]
+    res = kron.kron_mul_batch([(up(f), up(g)) for f, g in jobs], ctx=ctx)
+    for i, (x, (f, g)) in enumerate(zip(res, jobs)):
+        assert x["status"] == (kron.KR_ERR_DUP if i == 3 else 0)
+        if i != 3:
+            assert_poly_equal(x["exps"], x["coef"], oracle.poly_mul(f, g), f"job {i}")
