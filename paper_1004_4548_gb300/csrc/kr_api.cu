@@ -644,14 +644,15 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
         WinOut& O = Z.wout[k];
         const int64_t nw = k ? win_cap_total - win_cap_total1 : win_cap_total1;
         int64_t terms = 0;
-        for (int p : win_ids[k]) terms += plans[p].out_cap;
+        double windows = 0.0;
+        for (int p : win_ids[k]) {
+          terms += plans[p].out_cap;
+          windows += (double)plans[p].p.win.nw;
+        }
         O.cap = terms;
         O.key = b.take<uint64_t>(terms);
         O.val = b.take<uint64_t>(terms);
-        // pieces: a window whose keys cluster is halved down to each cluster, up to
-        // about 20 (32-bit offsets) or 36 times (64-bit), and a cluster that fills
-        // a table takes more than half the pairs of a window
-        O.nseg = nw ? std::min(ctx->win_pieces, (k ? 40 : 16) * nw + 4096) : 0;
+        O.nseg = nw ? std::min(ctx->win_pieces, win_pieces(windows)) : 0;
         O.seg = b.take<WinSeg>(O.nseg);
       }
       Z.wstage = b.take<unsigned char>((int64_t)win_staging(win_stage, ctx->num_sms));

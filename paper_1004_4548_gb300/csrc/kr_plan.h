@@ -44,6 +44,16 @@ constexpr double WIN_BOUND_BYTES = 16.0 * 1024 * 1024 * 1024;
 // output room per estimated term: +10% is about six standard errors of the
 // 4096-register HyperLogLog
 constexpr double WIN_ROOM = 1.1;
+// room for the pieces of `windows` planned windows: one a window and two where it
+// does not fit a list, more where keys cluster (a window is halved down to each
+// cluster, up to about 50 times for 64-bit offsets).  A product that takes more
+// goes through the table.  Kept to the 32-bit indices of the pieces; 64 bytes a
+// window, against 32 KB for a window's terms.
+constexpr int64_t win_pieces(double windows) {
+  return windows < 5e8 ? 4 * (int64_t)windows + 65536 : INT32_MAX;
+}
+static_assert(win_pieces(WIN_MAX_WALK * WIN_MAX_LIST / (0.49 * WIN_SLOTS_64)) < INT32_MAX,
+              "the largest product's pieces have 32-bit indices");
 constexpr int HASH_TILE_I = 32;
 constexpr int HASH_TILE_J = 1024;
 
