@@ -1269,7 +1269,10 @@ struct WinRun {
     const int64_t* start = P.win.start + wfirst;
     const bool narrow = sizeof(KT) == 8 || start[m] - start[0] <= (int64_t)0xfffffff0ll;   // offsets fit
     const bool sparse = narrow && (P.win.merge ? win_distinct(D, wfirst, D.nw) > 0.5f : P.win.sparse != 0);
-    const bool staged = sparse && P.win.stage && m > 1 && m <= WST;
+    // (the staging area holds Win::stage windows, at most WST; a run that starts where keys
+    // are distinct may go on into a region where they are not, whose windows are
+    // weighed otherwise)
+    const bool staged = sparse && m > 1 && m <= min(P.win.stage, WST);
     const bool listed = sparse && m == 1 && start[1] - start[0] > SLOTS;
     if (staged) stage(D, start, soff, sval);
     const int parts = staged ? (int)m : 1;

@@ -233,3 +233,19 @@ def test_terms_in_any_order(kron, n):
     with pytest.raises(kron.KronError) as err:
         poly(kron, one, Poly(np.ascontiguousarray(e), coef))
     assert err.value.status == kron.KR_ERR_DUP
+
+
+def test_runs_across_regions(kron):
+    """Keys shared in one part of the range and distinct in the others, so that runs of both kinds meet."""
+    rng = Rng(81)
+
+    def both(which, seed):
+        a, b = mp_sparse(which, 9, -1000, 1000, seed), random_poly(5, 2700, 0, 45, seed + 1)
+        e = np.concatenate([a.exps, b.exps + np.array([[0], [0], [0], [0], [200]], np.int32)], axis=1)
+        p = rng.perm(e.shape[1])
+        return Poly(np.ascontiguousarray(e[:, p]), np.concatenate([a.coef, b.coef])[p])
+
+    f, g = both("f", 82), both("g", 84)
+    a = [to_np(x) for x in poly(kron, f, g)[:2]]
+    b = [to_np(x) for x in poly(kron, f, g, table_slots=1 << 26)[:2]]
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
