@@ -457,7 +457,7 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
   std::vector<int32_t> h_hll_local;
   for (int p : hll_ids) h_hll_local.push_back(local[p]);
   std::vector<int32_t> h_win_local;
-  int64_t win_cap_total = 0, win_cap_total1 = 0, win_max_terms = 0, win_max_samples = 0, win_max_bins = 0;
+  int64_t win_cap_total = 0, win_cap_total1 = 0, win_max_terms = 0, win_max_samples = 0, win_max_bins = 0, win_max_windows = 0;
   bool win_poisson = false;
   std::vector<int> win_merge[2];   // merging products, by position in their kind's list
   int win_stage = 0;
@@ -470,6 +470,7 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       win_max_terms = std::max(win_max_terms, std::max(P.f.n, P.g.n));
       win_max_samples = std::max(win_max_samples, P.win.samples);
       win_max_bins = std::max(win_max_bins, P.win.nbins);
+      win_max_windows = std::max(win_max_windows, P.win.nw);
       win_poisson |= P.nt > 0;
       if (P.win.merge) {
         const int k = P.win.kind - 1;
@@ -871,7 +872,7 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     for (int k = 0, at = 0; k < 2; at += (int)win_ids[k].size(), ++k) {
       if (win_ids[k].empty()) continue;
       ck(ctx, launch_win_plan(A.lprods, A.win_ids + at, (int)win_ids[k].size(), win_poisson,
-                              win_merge[k].data(), (int)win_merge[k].size(), win_max_terms, win_max_samples, win_max_bins, A.win_prefix[k], k ? WIN_SLOTS_64 : WIN_SLOTS_32,
+                              win_merge[k].data(), (int)win_merge[k].size(), win_max_terms, win_max_samples, win_max_bins, win_max_windows, A.win_prefix[k], k ? WIN_SLOTS_64 : WIN_SLOTS_32,
                               (int64_t)ctx->num_sms * WIN_CTAS_PER_SM, A.win_done + k, s),
          "window plan");
       ctx->launches += 3 + (win_poisson ? 1 : 0) + (win_merge[k].empty() ? 0 : 1 + (int)win_merge[k].size());
@@ -889,6 +890,13 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       pl.p.f.nkeep = hl[q].f.nkeep;
       pl.p.g.nkeep = hl[q].g.nkeep;
     }
+    bool refused = false;   // by the window planning
+    for (int q = 0; q < nlive; ++q)
+      if (hl[q].status == ST_WINDOW) {
+        ctx->win_off[live_ids[q]] = 1;
+        refused = true;
+      }
+    if (refused) return false;
   }
   if (ctx->split_hist) {
     // kron_split_hist: sample the output keys of the (one) product and stop
@@ -916,11 +924,14 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     Bump hb2 = (ctx->replay || deferred) ? hb : Bump(ctx->pinned);
     Prod* hl2 = hb2.take<Prod>(nlive);
     if (!deferred) {   // a deferred product's phase B2 plan went up with phase B1's
-      for (int q = 0; q < nlive; ++q) {
-        hl2[q] = plans[live_ids[q]].p;
-        hl2[q].nout = 0;   // (as a repeated phase's plans hold the counts of the attempt before)
+      // (and a replay's: its phase B1 may also have found that a product no longer fits its plan)
+      if (!ctx->replay) {
+        for (int q = 0; q < nlive; ++q) {
+          hl2[q] = plans[live_ids[q]].p;
+          hl2[q].nout = 0;   // (a repeated phase's plans hold the counts of the attempt before)
+        }
+        ck(ctx, cudaMemcpyAsync(A.lprods, hl2, sizeof(Prod) * nlive, cudaMemcpyHostToDevice, s), "upload plan");
       }
-      ck(ctx, cudaMemcpyAsync(A.lprods, hl2, sizeof(Prod) * nlive, cudaMemcpyHostToDevice, s), "upload plan");
       int64_t* st = hb2.take<int64_t>(nlive + 1);
       memcpy(st, h_chunk_begin.data(), 8 * (size_t)(nlive + 1));
       ck(ctx, cudaMemcpyAsync(Z.chunk_begin, st, 8 * (size_t)(nlive + 1), cudaMemcpyHostToDevice, s),
@@ -1034,7 +1045,6 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
     bool retry = false, refused = false;
     for (int q = 0; q < nlive; ++q) {
       const int p = live_ids[q];
-      // (a replay's upload is captured: hl2 stays as it was uploaded)
       const Prod& P = ctx->replay ? plans[p].p : hl2[q];
       plans[p].p.nout = P.nout;
       plans[p].p.out_start = P.out_start;

@@ -573,9 +573,9 @@ cudaError_t launch_hash_insert(Prod* dprods, const int32_t* dhash_prods, const i
 // Windowed accumulation: lists, bucket indexes, histogram and cuts of every
 // listed product (drprefix: nwp + 1 offsets of runs; ddone: a zeroed counter;
 // merging: positions in the list of the `merge` products with Win::merge).
-cudaError_t launch_win_plan(const Prod* dprods, const int32_t* dwprods, int nwp, bool poisson,
+cudaError_t launch_win_plan(Prod* dprods, const int32_t* dwprods, int nwp, bool poisson,
                             const int* merging, int merge,
-                            int64_t max_terms, int64_t max_samples, int64_t max_bins, int64_t* drprefix,
+                            int64_t max_terms, int64_t max_samples, int64_t max_bins, int64_t max_windows, int64_t* drprefix,
                             int64_t slots, int64_t ctas, unsigned int* ddone, cudaStream_t s);
 // The windows of the listed products of one kind.
 struct WinLaunch {

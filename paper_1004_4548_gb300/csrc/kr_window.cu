@@ -146,7 +146,8 @@ __global__ void __launch_bounds__(256) k_win_lists(const Prod* __restrict__ prod
 }
 
 // Bucket index of every searched list and, by one thread per list, the list's
-// and the product's descriptors.
+// and the product's descriptors.  The buckets of a wide gap (a far term's, all
+// 65536 of them) are written by the whole warp.
 __global__ void __launch_bounds__(256) k_win_index(const Prod* __restrict__ prods,
                                                    const int32_t* __restrict__ wprods) {
   const Prod& P = prods[wprods[blockIdx.y >> 1]];
@@ -181,11 +182,23 @@ __global__ void __launch_bounds__(256) k_win_index(const Prod* __restrict__ prod
   L.shift = sh;
   L.nidx = (L.span >> sh) + 1;
   int32_t* idx = (int32_t*)L.idx;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j <= L.n;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t blo = j == 0 ? 0 : max((L.code[j - 1] >> sh) + 1, (int64_t)0);
-    const int64_t bhi = j == L.n ? L.nidx : min(L.code[j] >> sh, L.nidx);
-    for (int64_t b = blo; b <= bhi; ++b) idx[b] = (int32_t)j;
+  const int lane = threadIdx.x & 31;
+  for (int64_t j0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; j0 <= L.n;
+       j0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t j = j0 + lane;
+    int blo = 1, bhi = 0;   // (at most 65536 buckets)
+    if (j <= L.n) {
+      blo = j == 0 ? 0 : (int)max((L.code[j - 1] >> sh) + 1, (int64_t)0);
+      bhi = j == L.n ? (int)L.nidx : (int)min(L.code[j] >> sh, L.nidx);
+    }
+    unsigned wide = __ballot_sync(WFULL, bhi - blo >= 32);
+    if (bhi - blo < 32)
+      for (int b = blo; b <= bhi; ++b) idx[b] = (int32_t)j;
+    for (; wide; wide &= wide - 1) {
+      const int src = __ffs(wide) - 1;
+      const int lo = __shfl_sync(WFULL, blo, src), hi = __shfl_sync(WFULL, bhi, src);
+      for (int b = lo + lane; b <= hi; b += 32) idx[b] = (int32_t)(j0 + src);
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     D.L[which] = L;
@@ -203,7 +216,9 @@ __device__ __forceinline__ uint32_t hash32(uint64_t x) { return (uint32_t)(mix64
 
 // Histogram of the output keys of `samples` term pairs (all of them when
 // samples is the number of pairs; else stratified over A, B's term by a
-// counter-based hash).
+// counter-based hash).  A warp adds up the hits of its first lane's bin until that
+// changes: where one bin takes nearly all samples, the adds of 5.4 million one by one
+// took 4.3 ms.
 __global__ void __launch_bounds__(256) k_win_hist(const Prod* __restrict__ prods,
                                                   const int32_t* __restrict__ wprods) {
   const Prod& P = prods[wprods[blockIdx.y]];
@@ -218,38 +233,157 @@ __global__ void __launch_bounds__(256) k_win_hist(const Prod* __restrict__ prods
   const int sh = P.win.bin_shift;
   const uint64_t K0 = (uint64_t)P.klo, K = (uint64_t)P.kspan;
   const int64_t last = P.win.nbins - 1;
-  auto hit = [&](int64_t key) {
-    const uint64_t k = (uint64_t)key - K0;
-    if (k < K) atomicAdd(&P.win.hist[min((int64_t)(k >> sh), last)], 1u);
+  const int lane = threadIdx.x & 31;
+  int cur = -1;   // the bin being added up (of the whole warp), and its hits
+  uint32_t hits = 0;
+  auto flush = [&]() {
+    if (lane == 0 && cur >= 0) atomicAdd(&P.win.hist[cur], hits);
   };
-  for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < S;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    int64_t i, j;
+  auto hit = [&](bool act, int64_t key) {   // by whole warps
+    const uint64_t k = (uint64_t)key - K0;
+    act = act && k < K;
+    const int bin = act ? (int)min((int64_t)(k >> sh), last) : -1, first = __shfl_sync(WFULL, bin, 0);
+    if (act && bin != first) atomicAdd(&P.win.hist[bin], 1u);
+    if (first != cur) {
+      flush();
+      cur = first;
+      hits = 0;
+    }
+    hits += (uint32_t)__popc(__ballot_sync(WFULL, bin == first));
+  };
+  for (int64_t u0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; u0 < S;
+       u0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t u = u0 + lane;
+    bool act = u < S;
+    int64_t i = 0, j = 0;
     if (all) {
       i = u / G.n;
       j = u - i * G.n;
-      if (i >= nf || j >= ng) continue;
-    } else {
+      act = act && i < nf && j < ng;
+      if (!act) i = j = 0;
+    } else if (act) {
       i = (int64_t)((uint64_t)u * (uint64_t)nf / (uint64_t)S);   // samples < 2^32, terms < 2^31
       j = (int64_t)(((uint64_t)hash32((uint64_t)u + 1ull) * (uint64_t)ng) >> 32);
     }
     const int64_t pc = F.code[i] + G.code[j];
     if (P.nt == 0) {
-      hit(pc);
+      hit(act, pc);
       continue;
     }
     const int kd = F.kind[i] ^ G.kind[j];
     const int64_t ts = F.tcode[i] + G.tcode[j];
     int64_t td = F.tcode[i] - G.tcode[j];
     if (td < 0) td = -td;
-    hit(kd * T2Wp + ts * P.Wp + pc);
-    if (!(td == 0 && kd)) hit(kd * T2Wp + td * P.Wp + pc);
+    hit(act, kd * T2Wp + ts * P.Wp + pc);
+    hit(act && !(td == 0 && kd), kd * T2Wp + td * P.Wp + pc);
   }
+  flush();
 }
 
 // One CTA per product: the windows' starts, from the histogram.  The last CTA
 // to finish turns the products' window counts into offsets.
+//
+// A bin's windows lie as if its samples were spread evenly, which is wrong by at
+// most the bin's own windows.  Where a bin holds more of them than a CTA's share
+// of all (a cluster in a range that a few far terms made wide: 1820 terms of a
+// simplex and one monomial of degree 10^9, squared, lie in one bin of 6601), the
+// cuts are quantiles of sampled keys instead, found by sorting the sample here.
+// With the bins alone one CTA formed most of the pairs, halving its windows again
+// and again: 18.7 ms for those 3.3 M pairs, now 0.37 (a table in device memory
+// 0.69); 583 ms for 9 M pairs of 3.8 M keys, now 0.90 (1.47).  Keys so close that
+// not even quantiles divide them (25 M pairs on 10000 keys) are left to the table,
+// which adds them from all CTAs at once.
 constexpr int WC_THREADS = 1024;
+constexpr int WC_SORT = 16 * WC_THREADS;  // sampled keys at most (128 KB)
+__host__ __device__ inline int wc_sort_size(int64_t windows) {   // a power of two
+  int n = 2 * WC_THREADS;
+  while (n < WC_SORT && n < 4 * windows) n <<= 1;
+  return n;
+}
+constexpr int64_t WC_CROWD = 8;          // windows in a bin that are few in any case
+constexpr int64_t WC_DIRECT = 512;       // windows' pairs on the keys of one directly addressed window at most:
+                                         // an update takes about 0.3 ns there, a table's call 0.5 ms at least
+
+// The key, relative to klo, of sample u of n term pairs (-1: outside the range).
+__device__ __forceinline__ int64_t wc_sample(const Prod& P, int64_t u, int64_t n) {
+  const Operand& F = P.win.swap ? P.g : P.f;
+  const Operand& G = P.win.swap ? P.f : P.g;
+  const int64_t i = u * F.nkeep / n;
+  // multiples of the golden ratio: spread over G evenly for any number of samples
+  const int64_t j = (int64_t)(((uint64_t)((uint32_t)u * 2654435769u) * (uint64_t)G.nkeep) >> 32);
+  int64_t key = F.code[i] + G.code[j];
+  if (P.nt) {
+    const int kd = F.kind[i] ^ G.kind[j];
+    int64_t T = F.tcode[i] + ((hash32((uint64_t)u + 77ull) & 1u) ? G.tcode[j] : -G.tcode[j]);
+    if (T < 0) T = -T;
+    if (T == 0 && kd) return -1;
+    key += kd * (P.T2 * P.Wp) + T * P.Wp;
+  }
+  key -= P.klo;
+  return key >= 0 && key < P.kspan ? key : -1;
+}
+
+// Sorts the CTA's words, E a thread in sequence (v[e] is word E t + e), by a
+// bitonic network: strides below E within the thread, below 32 E by shuffles, the
+// others through shared memory k.  (Every step through shared memory took 400 us for
+// 16384 words.)
+template <int E>
+__device__ __forceinline__ void wc_sort(uint64_t (&v)[E], uint64_t* k) {
+  const int tid = threadIdx.x;
+  constexpr int N = E * WC_THREADS;
+  for (int size = 2; size <= N; size <<= 1) {
+    for (int stride = size >> 1; stride >= E; stride >>= 1) {
+      const int far = stride / E;   // the partner's distance in threads
+      const bool low = (((tid * E) & size) == 0) == ((tid & far) == 0);   // keeps the smaller word
+      if (far >= 32) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) k[e * WC_THREADS + tid] = v[e];
+        __syncthreads();
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const uint64_t o = far >= 32 ? k[e * WC_THREADS + (tid ^ far)] : __shfl_xor_sync(WFULL, v[e], far);
+        v[e] = (o < v[e]) == low ? o : v[e];
+      }
+      if (far >= 32) __syncthreads();
+    }
+#pragma unroll
+    for (int stride = E / 2; stride > 0; stride >>= 1)
+      if (stride < size) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (!(e & stride)) {
+            const uint64_t a = v[e], b = v[e | stride];
+            const bool swap = (a > b) == (((tid * E + e) & size) == 0);
+            v[e] = swap ? b : a;
+            v[e | stride] = swap ? a : b;
+          }
+      }
+  }
+}
+
+// E * WC_THREADS sampled keys into k, ascending; returns how many lie in range (the first ones).
+template <int E>
+__device__ __noinline__ int wc_sorted_sample(const Prod& P, uint64_t* k) {
+  uint64_t v[E];
+  int valid = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {   // (in any order)
+    const int64_t x = wc_sample(P, e * WC_THREADS + threadIdx.x, E * WC_THREADS);
+    v[e] = (uint64_t)x;   // (-1 sorts last)
+    valid += x >= 0;
+  }
+  __shared__ int s_valid;
+  if (threadIdx.x == 0) s_valid = 0;
+  __syncthreads();
+  valid = __reduce_add_sync(WFULL, valid);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&s_valid, valid);
+  wc_sort<E>(v, k);
+#pragma unroll
+  for (int e = 0; e < E; ++e) k[threadIdx.x * E + e] = v[e];
+  __syncthreads();
+  return s_valid;
+}
 
 __device__ __forceinline__ int64_t wc_scan(int64_t v, int64_t* total, int64_t* ws) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -309,19 +443,27 @@ __device__ __forceinline__ float win_distinct(const WinDesc& D, int64_t w, int64
   return n >= 4.0f ? D.rs[r] / n : 1.0f;
 }
 
-__global__ void __launch_bounds__(WC_THREADS) k_win_cut(const Prod* __restrict__ prods,
+__global__ void __launch_bounds__(WC_THREADS) k_win_cut(Prod* __restrict__ prods,
                                                         const int32_t* __restrict__ wprods, int nwp,
-                                                        int64_t* __restrict__ rprefix, int64_t slots,
+                                                        int64_t* __restrict__ rprefix, int64_t slots, int64_t ctas,
                                                         unsigned int* __restrict__ done) {
-  extern __shared__ uint32_t hs[];   // the histogram, one word of padding per 32 bins
+  extern __shared__ __align__(8) uint32_t hs[];   // the histogram, one word of padding per 32 bins; or sampled keys
   __shared__ int64_t ws[WC_THREADS / 32];
-  __shared__ unsigned int s_last;
-  const Prod& P = prods[wprods[blockIdx.x]];
+  __shared__ unsigned int s_last, s_top;
+  Prod& P = prods[wprods[blockIdx.x]];
   int64_t nw = 1;
   if (P.status == 0) {
     const int nb = (int)P.win.nbins;
-    for (int i = threadIdx.x; i < nb; i += WC_THREADS) hs[i + (i >> 5)] = P.win.hist[i];
+    uint32_t top = 0;
+    if (threadIdx.x == 0) s_top = 0;
+    for (int i = threadIdx.x; i < nb; i += WC_THREADS) {
+      const uint32_t x = P.win.hist[i];
+      hs[i + (i >> 5)] = x;
+      top = max(top, x);
+    }
     __syncthreads();
+    top = __reduce_max_sync(WFULL, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);   // (read after the scan's barriers)
     // inclusive prefix sums in place
     const int per = (nb + WC_THREADS - 1) / WC_THREADS;
     const int a = min(nb, per * (int)threadIdx.x), b = min(nb, a + per);
@@ -335,11 +477,32 @@ __global__ void __launch_bounds__(WC_THREADS) k_win_cut(const Prod* __restrict__
     // bin as if the bin's samples were spread evenly, at a multiple of an eighth
     // of `slots` keys from the bin's start (bins are at least `slots` wide):
     // windows that would start at the same key are one
-    const int64_t spw = max((int64_t)1, (tot + P.win.nw - 1) / max((int64_t)1, P.win.nw));
-    const int64_t nk = max((int64_t)1, (tot + spw - 1) / spw);
+    int64_t spw = max((int64_t)1, (tot + P.win.nw - 1) / max((int64_t)1, P.win.nw));
+    int64_t nk = max((int64_t)1, (tot + spw - 1) / spw);
     const float binw = (float)(int64_t(1) << P.win.bin_shift);
+    // a CTA's share, and a quarter more: the 6188 x 6188 weighted product (34 of 9539
+    // windows in a bin, a share of 31) is cut well by its bins
+    const bool crowded = (int64_t)s_top > spw * max(WC_CROWD, 5 * nk / (4 * ctas));   // uniform
+    const uint64_t* const ks = (const uint64_t*)hs;
+    int64_t nv = 0;   // sampled keys
+    if (crowded) {
+      __syncthreads();   // the histogram has been read
+      const int n = wc_sort_size(P.win.nw);
+      uint64_t* const k = (uint64_t*)hs;
+      nv = n == 2 * WC_THREADS ? wc_sorted_sample<2>(P, k) : n == 4 * WC_THREADS ? wc_sorted_sample<4>(P, k)
+         : n == 8 * WC_THREADS ? wc_sorted_sample<8>(P, k) : wc_sorted_sample<16>(P, k);
+      nk = P.win.nw;
+      spw = 1;   // (Win::before counts windows)
+      tot = nk;
+    }
     auto start_of = [&](int64_t k) -> int64_t {   // relative to klo
       if (k <= 0) return 0;
+      if (crowded) {
+        const double x = (double)k * (double)nv / (double)nk;
+        const int64_t i = min((int64_t)x, nv);
+        const int64_t lo = i > 0 ? (int64_t)ks[i - 1] : 0, hi = i < nv ? (int64_t)ks[i] : P.kspan;
+        return (lo + min((int64_t)((x - (double)i) * (double)(hi - lo)), hi - lo)) & ~(slots / 8 - 1);
+      }
       const uint32_t want = (uint32_t)(k * spw);
       int lo = 0, hi = nb - 1;   // the first bin whose prefix exceeds it
       while (lo < hi) {
@@ -377,6 +540,12 @@ __global__ void __launch_bounds__(WC_THREADS) k_win_cut(const Prod* __restrict__
     }
     if (!P.win.merge)
       for (int64_t q = threadIdx.x; q <= nw; q += WC_THREADS) P.win.run[q] = (int32_t)q;
+    if (crowded) {   // windows that would start at the same key are one: too many pairs for a CTA?
+      __syncthreads();
+      uint32_t most = 0;
+      for (int64_t q = threadIdx.x; q < nw; q += WC_THREADS) most = max(most, P.win.before[q + 1] - P.win.before[q]);
+      if ((int64_t)most > max(WC_DIRECT, 16 * nk / ctas)) atomicOr(&P.status, ST_WINDOW);
+    }
   }
   if (done) win_prefix(nw, nwp, rprefix, done, ws, &s_last);
 }
@@ -1593,8 +1762,9 @@ __global__ void __launch_bounds__(256) k_win_dup(const Prod* __restrict__ prods,
   }
 }
 
-cudaError_t launch_win_plan(const Prod* dprods, const int32_t* dwprods, int nwp, bool poisson, const int* merging, int merge,
-                            int64_t max_terms, int64_t max_samples, int64_t max_bins, int64_t* drprefix, int64_t slots, int64_t ctas,
+cudaError_t launch_win_plan(Prod* dprods, const int32_t* dwprods, int nwp, bool poisson, const int* merging, int merge,
+                            int64_t max_terms, int64_t max_samples, int64_t max_bins, int64_t max_windows, int64_t* drprefix,
+                            int64_t slots, int64_t ctas,
                             unsigned int* ddone, cudaStream_t s) {
   if (nwp <= 0) return cudaSuccess;
   auto gx = [](int64_t n, int64_t most) {
@@ -1605,10 +1775,10 @@ cudaError_t launch_win_plan(const Prod* dprods, const int32_t* dwprods, int nwp,
   k_win_index<<<dim3(gx(2 * max_terms, 64), 2 * nwp), 256, 0, s>>>(dprods, dwprods);
   const int64_t most = nwp > 64 ? 32 : 2048 / nwp;
   k_win_hist<<<dim3(gx(max_samples, most), nwp), 256, 0, s>>>(dprods, dwprods);
-  const size_t smem = (size_t)(max_bins + max_bins / 32 + 1) * 4;
+  const size_t smem = std::max((size_t)(max_bins + max_bins / 32 + 1) * 4, (size_t)wc_sort_size(max_windows) * 8);
   cudaError_t e = raise_smem_limit((const void*)k_win_cut, smem);
   if (e != cudaSuccess) return e;
-  k_win_cut<<<nwp, WC_THREADS, smem, s>>>(dprods, dwprods, nwp, drprefix, slots, merge ? nullptr : ddone);
+  k_win_cut<<<nwp, WC_THREADS, smem, s>>>(dprods, dwprods, nwp, drprefix, slots, ctas, merge ? nullptr : ddone);
   if (merge) {
     for (int i = 0; i < merge; ++i) k_win_dup<<<WIN_DUP_SAMPLES, 256, 0, s>>>(dprods, dwprods + merging[i]);
     k_win_runs<<<nwp, WC_THREADS, 0, s>>>(dprods, dwprods, nwp, drprefix, slots, ctas, ddone);
