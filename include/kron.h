@@ -455,8 +455,10 @@ kr_status kr_selftest_bounded_wait(int32_t device);
  * KR_LIMIT_WINDOW_ROOM: output room per estimated term (below 1 the estimate is
  *   always short)
  * KR_LIMIT_WINDOW_PIECES: stretches of terms that the windows of a call may put
- *   down (a product that needs more is done again by the table) */
-enum { KR_LIMIT_WINDOW_BYTES = 0, KR_LIMIT_WINDOW_ROOM = 1, KR_LIMIT_WINDOW_PIECES = 2 };
+ *   down (a product that needs more is done again by the table)
+ * KR_LIMIT_GROWTHS: how many of the next growths of the accumulators' scratch
+ *   fail as if device memory had run out */
+enum { KR_LIMIT_WINDOW_BYTES = 0, KR_LIMIT_WINDOW_ROOM = 1, KR_LIMIT_WINDOW_PIECES = 2, KR_LIMIT_GROWTHS = 3 };
 kr_status kr_selftest_limit(kr_ctx* ctx, int32_t which, double value);
 
 #ifdef __cplusplus

@@ -13,5 +13,6 @@ from .binding import (  # noqa: F401
     kron_plan, kron_encode, kron_decode, poly_mul, poisson_mul, kr_probe_smem_atomic_rate,
     kr_probe_smem_accumulate_rate, kr_probe_table_update_rate, kr_probe_alu_rate,
     kr_selftest_bounded_wait, kr_selftest_limit, KR_LIMIT_WINDOW_BYTES, KR_LIMIT_WINDOW_ROOM, KR_LIMIT_WINDOW_PIECES,
+    KR_LIMIT_GROWTHS,
     kron_dense_product_static, kron_mul_batch, PreparedBatch,
 )

@@ -372,7 +372,7 @@ def kr_selftest_bounded_wait(device: int = 0) -> int:
     return int(load().kr_selftest_bounded_wait(device))
 
 
-KR_LIMIT_WINDOW_BYTES, KR_LIMIT_WINDOW_ROOM, KR_LIMIT_WINDOW_PIECES = 0, 1, 2
+KR_LIMIT_WINDOW_BYTES, KR_LIMIT_WINDOW_ROOM, KR_LIMIT_WINDOW_PIECES, KR_LIMIT_GROWTHS = 0, 1, 2, 3
 
 
 def kr_selftest_limit(ctx: Context, which: int, value: float = 0.0):

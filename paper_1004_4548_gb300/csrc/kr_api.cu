@@ -86,6 +86,10 @@ struct kr_ctx {
   // is settled)
   std::vector<char> win_off;
   bool win_refused = false;
+  // how a call that ran out of memory with windows runs again: 0 room by the
+  // bound on the terms, 1 by their estimate, 2 without windows
+  int win_mode = 0;
+  int fail_growths = 0;   // self-test: growths of the accumulators' arena that fail
   // stage timing (CUDA events on the call's stream) and launch counting
   bool profile = false;
   std::vector<cudaEvent_t> ev;
@@ -161,6 +165,10 @@ void ensure(kr_ctx* ctx, void** buf, size_t* cap, size_t need, cudaStream_t s) {
   if (*buf) cudaFree(*buf);
   *buf = nullptr;
   *cap = 0;
+  if (buf == &ctx->acc && ctx->fail_growths > 0) {
+    --ctx->fail_growths;
+    ck(ctx, cudaErrorMemoryAllocation, "scratch growth");
+  }
   size_t want = need + need / 4 + (1 << 20);
   ck(ctx, cudaMalloc(buf, want), "cudaMalloc scratch");
   *cap = want;
@@ -426,7 +434,7 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
       win_bound += 32.0 * std::min((plans[p].p.nt > 0 ? 2.0 : 1.0) * (double)plans[p].p.f.n * (double)plans[p].p.g.n,
                                    (double)plans[p].p.kspan);
   }
-  const bool win_estimate = win_bound > ctx->win_bound;
+  const bool win_estimate = ctx->win_mode > 0 || win_bound > ctx->win_bound;
   for (int p = 0; p < nprod; ++p) {
     if (plans[p].st != KR_OK) continue;
     if (plans[p].empty) {   // truncated to nothing: a zero product
@@ -1139,6 +1147,28 @@ bool run_pipeline(kr_ctx* ctx, const std::vector<JobIn>& ins, cudaStream_t s,
   }
 }
 
+// After running out of memory: whether the call can run again with less of it,
+// its windows' room estimated, then without windows.  (Room by the bound on the
+// terms is up to 32 bytes a term pair; a table takes about 64 a term.)
+bool shrink_windows(kr_ctx* ctx, size_t nprod, cudaStream_t s) {
+  bool any = false;
+  for (const Plan& pl : ctx->plans) any |= pl.st == KR_OK && !pl.empty && pl.p.win.kind != 0;
+  if (!any || ctx->win_mode >= 2) return false;
+  ck(ctx, cudaStreamSynchronize(s), "sync before scratch release");
+  if (ctx->acc) cudaFree(ctx->acc);
+  ctx->acc = nullptr;
+  ctx->acc_cap = 0;
+  ctx->nev = 0;
+  if (++ctx->win_mode == 2) ctx->win_off.assign(nprod, 1);
+  return true;
+}
+
+// A run of the pipeline that nothing has failed yet.
+void start_windows(kr_ctx* ctx, size_t nprod) {
+  ctx->win_mode = 0;
+  ctx->win_off.assign(nprod, 0);
+}
+
 struct CtxGuard {
   kr_ctx* c;
   int prev = -1;
@@ -1196,7 +1226,7 @@ void join_raw(kr_ctx* ctx, cudaStream_t s) {
 
 kr_status emit_poly(kr_ctx* ctx, kr_poly_out* h, cudaStream_t s) {
   const Prod& P = ctx->res_prod;
-  const int64_t n = ctx->res_n;
+  int64_t n = ctx->res_n;
   h->nterms = n;
   for (int k = 0; k < KR_MAXV; ++k) { h->omin[k] = 0; h->omax[k] = 0; }
   for (int k = 0; k < P.np; ++k) {
@@ -1230,7 +1260,13 @@ kr_status emit_poly(kr_ctx* ctx, kr_poly_out* h, cudaStream_t s) {
       if (st != KR_OK) return st;
       return ctx->res_n > h->capacity ? KR_ERR_CAPACITY : KR_OK;
     }
-    join_raw(ctx, s);
+    if (n < 0) {   // (scratch for the terms there are: the bound on them may be many times more)
+      const kr_status st = settle_deferred(ctx, s);
+      h->nterms = n = st == KR_OK ? ctx->res_n : 0;
+      if (st != KR_OK) return st;
+      mark(ctx, s, "begin");
+    }
+    if (n <= h->capacity) join_raw(ctx, s);
   }
   if (n < 0) {
     const bool exps_dev = !h->exps || is_device_ptr(h->exps);
@@ -1398,7 +1434,7 @@ void keep_result(kr_ctx* ctx, const ProdResult& r, bool poisson) {
 template <typename Emit>
 kr_status run_single(kr_ctx* ctx, const JobIn& in, bool deferred, const DirectOut& direct, cudaStream_t s, Emit emit) {
   std::vector<ProdResult> res;
-  ctx->win_off.assign(1, 0);
+  start_windows(ctx, 1);
   for (;;) {
     ctx->allow_deferred = deferred;
     ctx->allow_raw = true;
@@ -1421,6 +1457,9 @@ kr_status run_single(kr_ctx* ctx, const JobIn& in, bool deferred, const DirectOu
       ctx->direct_done = false;
       if (!ctx->win_refused) return st;
       ctx->win_off[0] = 1;
+    } catch (const CudaFail& f) {
+      reset(true);
+      if (f.e != cudaErrorMemoryAllocation || !shrink_windows(ctx, 1, s)) throw;
     } catch (...) {
       reset(true);
       throw;
@@ -1546,6 +1585,7 @@ kr_status kr_selftest_limit(kr_ctx* ctx, int32_t which, double value) {
     case KR_LIMIT_WINDOW_BYTES: ctx->win_bound = value > 0.0 ? value : WIN_BOUND_BYTES; return KR_OK;
     case KR_LIMIT_WINDOW_ROOM: ctx->win_room = value > 0.0 ? value : WIN_ROOM; return KR_OK;
     case KR_LIMIT_WINDOW_PIECES: ctx->win_pieces = value > 0.0 ? (int64_t)value : INT64_MAX; return KR_OK;
+    case KR_LIMIT_GROWTHS: ctx->fail_growths = value > 0.0 ? (int)value : 0; return KR_OK;
   }
   return KR_ERR_INVALID;
 }
@@ -1777,11 +1817,10 @@ bool pseries_job_ok(const kr_pseries* f, const kr_pseries* g) {
 }
 
 // One wave of a batch: pipeline, then one batched decode into a fresh block.
-kr_status run_wave(kr_ctx* ctx, const std::vector<JobIn>& ins, const std::vector<int>& idx,
+kr_status try_wave(kr_ctx* ctx, const std::vector<JobIn>& ins, const std::vector<int>& idx,
                    kr_result* res, cudaStream_t s) {
   std::vector<ProdResult> pr;
   try {
-    ctx->win_off.assign(ins.size(), 0);
     while (!run_pipeline(ctx, ins, s, pr)) {}
   } catch (const CudaFail& f) {
     if (f.e == cudaErrorMemoryAllocation) {
@@ -1864,6 +1903,16 @@ kr_status run_wave(kr_ctx* ctx, const std::vector<JobIn>& ins, const std::vector
   ctx->launches += 1;
   ck(ctx, cudaStreamSynchronize(s), "sync decode");
   return KR_OK;
+}
+
+// (A wave of several products that runs out of memory is split by the caller.)
+kr_status run_wave(kr_ctx* ctx, const std::vector<JobIn>& ins, const std::vector<int>& idx,
+                   kr_result* res, cudaStream_t s) {
+  start_windows(ctx, ins.size());
+  for (;;) {
+    const kr_status st = try_wave(ctx, ins, idx, res, s);
+    if (st != KR_ERR_OOM || ins.size() > 1 || !shrink_windows(ctx, ins.size(), s)) return st;
+  }
 }
 
 }  // namespace
@@ -2019,15 +2068,24 @@ kr_status kron_batch_prepare(int32_t device, const kr_job* jobs, int32_t njobs, 
     if (b->ins.empty()) return KR_OK;
     // the prepared run
     std::vector<ProdResult> pr;
-    while (!run_pipeline(ictx, b->ins, s, pr)) {}
     std::vector<int> order;
-    for (int p = 0; p < (int)b->ins.size(); ++p)
-      if (pr[p].dprod) order.push_back(p);
-    std::sort(order.begin(), order.end(), [&](int a, int c) { return pr[a].dprod < pr[c].dprod; });
+    start_windows(ictx, b->ins.size());
+    for (;;) {
+      try {
+        while (!run_pipeline(ictx, b->ins, s, pr)) {}
+        order.clear();
+        for (int p = 0; p < (int)b->ins.size(); ++p)
+          if (pr[p].dprod) order.push_back(p);
+        std::sort(order.begin(), order.end(), [&](int a, int c) { return pr[a].dprod < pr[c].dprod; });
+        size_t bytes = sizeof(ResDesc) * (order.size() + 1) + 8 * (order.size() + 2) + 512;
+        for (int p : order) bytes += (size_t)pr[p].n * (4 * (pr[p].prod.np + pr[p].prod.nt) + 1 + 8) + 4 * 256;
+        ck(ictx, cudaMalloc(&b->block, bytes), "cudaMalloc results");
+        break;
+      } catch (const CudaFail& f) {
+        if (f.e != cudaErrorMemoryAllocation || !shrink_windows(ictx, b->ins.size(), s)) throw;
+      }
+    }
     const int nl = (int)order.size();
-    size_t bytes = sizeof(ResDesc) * (nl + 1) + 8 * (nl + 2) + 512;
-    for (int p : order) bytes += (size_t)pr[p].n * (4 * (pr[p].prod.np + pr[p].prod.nt) + 1 + 8) + 4 * 256;
-    ck(ictx, cudaMalloc(&b->block, bytes), "cudaMalloc results");
     Bump bb(b->block);
     b->d_rd = bb.take<ResDesc>(nl);
     b->d_ost = bb.take<int64_t>(nl + 1);
@@ -2185,7 +2243,7 @@ kr_status kron_split_hist(kr_ctx* ctx, const kr_job* job, int32_t nbins, int64_t
     ctx->split_nsamples = nsamples;
     ctx->split_seed = seed;
     ctx->split_hist = hist;
-    ctx->win_off.assign(1, 0);
+    start_windows(ctx, 1);
     std::vector<ProdResult> res;
     try {
       run_pipeline(ctx, {in}, s, res);

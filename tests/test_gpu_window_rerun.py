@@ -7,7 +7,8 @@ import pytest
 import oracle
 from tests.gpu_compare import assert_poly_equal, assert_pseries_close, to_np
 from tests.test_gpu_window import POLY, PSER, dev, poly, pseries
-from workloads import random_poly
+from tests.test_gpu_window_crowded import far
+from workloads import dense_total_degree, random_poly
 
 pytestmark = pytest.mark.gpu
 
@@ -115,3 +116,53 @@ def test_pieces_run_out(kron, limited):
         assert x["status"] == (kron.KR_ERR_DUP if i == 3 else 0)
         if i != 3:
             assert_poly_equal(x["exps"], x["coef"], oracle.poly_mul(f, g), f"job {i}")
+
+
+@pytest.mark.parametrize("failures", [1, 2, 3])
+def test_out_of_memory(kron, failures):
+    """A windowed product whose scratch does not fit runs again with estimated room, then through the table."""
+    import torch
+    f, g = POLY["shared_keys"]()
+    p, q = PSER["offsets_64"]()
+    r, rs = oracle.poly_mul(f, g), oracle.poisson_mul(p, q, keep_zero=True)
+    calls = {"poly": (lambda c: poly(kron, f, g, ctx=c), lambda o: assert_poly_equal(o[0], o[1], r)),
+             "host": (lambda c: poly(kron, f, g, ctx=c, host_out=True), lambda o: assert_poly_equal(o[0], o[1], r)),
+             "series": (lambda c: pseries(kron, p, q, ctx=c), lambda o: assert_pseries_close(o, rs)),
+             "batch": (lambda c: kron.kron_mul_batch([(up(f), up(g))], ctx=c, opts={"path": kron.KR_PATH_HASH}),
+                       lambda o: assert_poly_equal(o[0]["exps"], o[0]["coef"], r))}
+    for name, (call, check) in calls.items():
+        ctx = kron.Context()
+        kron.kr_selftest_limit(ctx, kron.KR_LIMIT_GROWTHS, failures)
+        if failures < 3:
+            check(call(ctx))
+        else:
+            with pytest.raises(kron.KronError) as err:
+                call(ctx)
+            assert err.value.status == kron.KR_ERR_OOM
+        check(call(ctx))   # the next call is not affected
+        ctx.close()
+    # several products: a wave is split before its products give up their windows
+    ctx = kron.Context()
+    kron.kr_selftest_limit(ctx, kron.KR_LIMIT_GROWTHS, failures)
+    for x in kron.kron_mul_batch([(up(f), up(g))] * 2, ctx=ctx):
+        assert x["status"] == 0
+        assert_poly_equal(x["exps"], x["coef"], r)
+    ctx.close()
+    torch.cuda.synchronize()
+
+
+def test_host_outputs_take_room_for_their_terms(kron):
+    """A product with far fewer terms than pairs, into host memory with room for every pair."""
+    f = far(dense_total_degree(4, 12, -1000, 1000, 61), 10 ** 9)
+    g = far(dense_total_degree(4, 11, -1000, 1000, 62), 10 ** 9)
+    r = oracle.poly_mul(f, g)
+    pairs = f.coef.size * g.coef.size
+    assert 50 * r.coef.size < pairs
+    ctx, base = kron.Context(), kron.Context()
+    ex, cf, _, _ = poly(kron, f, g, ctx=ctx, host_out=True, capacity=pairs)
+    assert_poly_equal(ex, cf, r)
+    poly(kron, f, g, ctx=base)
+    extra = ctx.scratch_bytes() - base.scratch_bytes()   # the decode's: 24 bytes a term, a quarter and 1 MB to spare
+    assert extra <= 1.25 * 24 * r.coef.size + (2 << 20)
+    ctx.close()
+    base.close()
