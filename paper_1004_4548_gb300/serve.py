@@ -10,10 +10,11 @@ interpreter lock) the dispatcher forms and starts the next batch on another
 worker, so the batches' work overlaps on the device.  Results stay on the
 device: each request gets its own copy of its product (torch tensors).
 
-The memory prediction per product is the term-product count times 16 bytes
-times the observed ratio of output terms to term-products (updated after
-every batch, separately for polynomials and Poisson series), plus the dense
-array or hash table it needs.
+The memory prediction per product is the larger of two: 64 bytes (dense array
+or hash table, ordering and output) for each of the output terms expected from
+the observed ratio of output terms to term-products (updated after every batch,
+separately for polynomials and Poisson series), and the room of a windowed
+product, 32 bytes for each of its updates whether or not they merge.
 
 A batch is also capped in work (term-products): the oldest waiting request
 always starts the batch, and later requests join it only while the cap holds,
@@ -42,6 +43,13 @@ from dataclasses import dataclass, field
 import numpy as np
 
 from . import binding as B
+
+# the library's limits of windowed products: room by the bound on the terms up to
+# here, staging areas from this many updates on and their size (32 windows for
+# each of 304 CTAs) at most
+WINDOW_BOUND = 16.0 * (1 << 30)
+STAGED_UPDATES = 8.0 * 600.0 * 2007
+STAGING_MOST = 304 * 32 * 7680 * 12.0
 
 
 @dataclass
@@ -143,7 +151,16 @@ class Server:
     def predict_bytes(self, r: Request) -> float:
         out_terms = r.pairs * self.ratio[r.poisson]
         # output (16 B) + ordering scratch (16 B) + table at load 0.5 (32 B) per term
-        return 64.0 * out_terms + 1e6
+        table = 64.0 * out_terms
+        # key windows: raw and ordered terms (32 B) by the bound on them, or by their
+        # estimate where the bound is large; a staging area for large products; the
+        # library grows its scratch by a quarter more than it needs
+        updates = (2.0 if r.poisson else 1.0) * r.pairs
+        room = 32.0 * updates if 32.0 * updates <= WINDOW_BOUND else 36.0 * out_terms
+        if updates > STAGED_UPDATES:
+            room += STAGING_MOST
+        terms = int(r.f.coef.shape[0]) + int(r.g.coef.shape[0])
+        return max(table, 1.25 * room) + 160.0 * terms + 8e6
 
     def _mul(self, w: _Worker, batch: list[Request], stream=None):
         stream = w.stream if stream is None else stream
