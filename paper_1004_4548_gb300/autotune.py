@@ -32,7 +32,8 @@ TABLE = os.path.join(HERE, "tuned.json")
 # memory per CTA is set by its largest block, so larger blocks would lower the
 # occupancy of every product in the batch
 DENSE_S = (2048, 4096, 8192)
-HASH_ALPHA = (0.3, 0.5, 0.7)
+# (windowed products, which these are, have no table that the load factor would size)
+HASH_ALPHA = (0.5,)
 
 _table_cache: dict | None = None
 

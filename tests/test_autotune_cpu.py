@@ -60,3 +60,15 @@ def test_lookup_guards():
     big = Poly(np.array([[0, 1 << 20], [0, 1 << 20], [0, 1 << 10]], np.int32), np.array([1, 2], np.int64))
     kb = at.class_key(at.features(big, big))
     assert at.opts_for(big, big, table={kb: {"path": 1, "block_slots": 4096}}) == {}
+
+
+def test_stored_table_is_of_the_present_candidates():
+    """A table measured against other choices than the present ones is stale."""
+    with open(at.TABLE) as fh:
+        t = json.load(fh)
+    assert t["candidates"] == {"dense_block_slots": list(at.DENSE_S), "hash_load_factor": list(at.HASH_ALPHA)}
+    assert len({json.dumps(c, sort_keys=True) for c in at.candidates({"poisson": True, "pairs": 1 << 20, "W": 1e12})}) == \
+        len(set(at.HASH_ALPHA)) == 1   # windowed products ignore the load factor: one hash candidate, not three alike
+    for key, o in t["classes"].items():
+        r = t["report"][key]
+        assert r["best"] == o and r["ms"] < 0.97 * r["default_ms"], key
