@@ -558,12 +558,35 @@ class _DevArray:
                                          "data": (int(ptr or 0), False), "version": 3, "strides": None}
 
 
+_VIEW_TYPES: dict = {}     # typestr -> (torch dtype, bytes)
+_VIEW_DEVICES: dict = {}
+_view_makers = None        # torch's constructors from a pointer, where this torch has them
+
+
 def _view(ptr, shape, typestr, device):
+    """A tensor of its own (storage, version counter) over library-owned device memory.  torch's constructors from a
+    pointer take 1.2 us an array, the array interface 1.7 and a parse of it; strided views of one tensor over a batch's
+    block take 0.9, but share its storage (saving or deep-copying one result takes the block) and its version counter
+    (changing one in place invalidates what autograd has saved of the others)."""
+    global _view_makers
     torch = _torch()
-    if not ptr or any(d == 0 for d in shape):
-        dt = {"<i4": torch.int32, "<i8": torch.int64, "<f8": torch.float64, "|u1": torch.uint8}[typestr]
-        return torch.empty(shape, dtype=dt, device=f"cuda:{device}")
-    return torch.as_tensor(_DevArray(ptr, shape, typestr), device=f"cuda:{device}")
+    if not _VIEW_TYPES:
+        _VIEW_TYPES.update({"<i4": (torch.int32, 4), "<i8": (torch.int64, 8), "<f8": (torch.float64, 8),
+                            "|u1": (torch.uint8, 1)})
+        makers = (getattr(torch._C, "_construct_storage_from_data_pointer", None),
+                  getattr(torch._C, "_construct_CUDA_Tensor_From_Storage_And_Metadata", None))
+        _view_makers = makers if all(makers) else False
+    dt, size = _VIEW_TYPES[typestr]
+    dev = _VIEW_DEVICES.get(device)
+    if dev is None:
+        dev = _VIEW_DEVICES.setdefault(device, torch.device("cuda", device))
+    if not ptr or 0 in shape:
+        return torch.empty(shape, dtype=dt, device=dev)
+    if not _view_makers:
+        return torch.as_tensor(_DevArray(ptr, shape, typestr), device=dev)
+    storage, tensor = _view_makers
+    return tensor({"size": shape, "stride": (shape[1], 1) if len(shape) == 2 else (1,), "dtype": dt, "storage_offset": 0},
+                  storage(ptr, dev, math.prod(shape) * size))
 
 
 def kron_split_hist(f, g, nbins: int = 65536, nsamples: int = 1 << 22, seed: int = 1,
@@ -639,50 +662,19 @@ _RES = np.dtype([("status", "<i4"), ("path", "<i4"), ("nterms", "<i8"), ("exps",
 assert _RES.itemsize == ctypes.sizeof(kr_result)
 
 
-class _Views:
-    """Views of library-owned device memory.  The arrays of a batch lie in one block (or a few): one
-    tensor over the block's bytes, and each result a strided view of it, costs a quarter of one tensor
-    per array (16 products: 0.1 ms instead of 0.4)."""
-
-    def __init__(self, sizes, device):
-        """sizes: (pointer, bytes) of every array; one base tensor where they are packed."""
-        self.device, self.base, self.typed = device, 0, None
-        if not sizes:
-            return
-        self.base = min(p for p, _ in sizes)
-        span = max(p + b for p, b in sizes) - self.base
-        if span > sum(b for _, b in sizes) + 512 * len(sizes) or any((p - self.base) % 8 for p, _ in sizes):
-            return   # several blocks
-        torch = _torch()
-        whole = _view(self.base, ((span + 7) // 8 * 8,), "|u1", self.device)
-        self.typed = {"<i4": (whole.view(torch.int32), 4), "<i8": (whole.view(torch.int64), 8),
-                      "<f8": (whole.view(torch.float64), 8), "|u1": (whole, 1)}
-
-    def get(self, ptr, shape, typestr):
-        if self.typed is None or not ptr or 0 in shape:
-            return _view(ptr, shape, typestr, self.device)
-        t, size = self.typed[typestr]
-        return t.as_strided(shape, (shape[1], 1) if len(shape) == 2 else (1,), (ptr - self.base) // size)
-
-
 def _results(jobs, res, n, device):
-    rows = np.frombuffer(res, _RES, n).tolist()
-    plan = []
-    for i, (status, path, m, exps, trig, kind, coef) in enumerate(rows):
-        job = jobs[i]
-        if job.kind == 1:
-            plan.append((("exps", exps, (job.pf.npoly, m), "<i4"), ("trig", trig, (job.pf.ntrig, m), "<i4"),
-                         ("kind", kind, (m,), "|u1"), ("coef", coef, (m,), "<f8")))
-        else:
-            plan.append((("exps", exps, (job.f.nvars, m), "<i4"),
-                         ("coef", coef, (m,), "<f8" if job.f.type == KR_F64 else "<i8")))
-    views = _Views([(ptr, math.prod(shape) * int(ts[2])) for p in plan for _, ptr, shape, ts in p
-                    if ptr and 0 not in shape], device)
     out = []
-    for (status, path, m, *_), p in zip(rows, plan):
+    for i, (status, path, m, exps, trig, kind, coef) in enumerate(np.frombuffer(res, _RES, n).tolist()):
+        job = jobs[i]
         d = {"status": status, "path": path, "nterms": m}
-        for name, ptr, shape, typestr in p:
-            d[name] = views.get(ptr, shape, typestr)
+        if job.kind == 1:
+            d["exps"] = _view(exps, (job.pf.npoly, m), "<i4", device)
+            d["trig"] = _view(trig, (job.pf.ntrig, m), "<i4", device)
+            d["kind"] = _view(kind, (m,), "|u1", device)
+            d["coef"] = _view(coef, (m,), "<f8", device)
+        else:
+            d["exps"] = _view(exps, (job.f.nvars, m), "<i4", device)
+            d["coef"] = _view(coef, (m,), "<f8" if job.f.type == KR_F64 else "<i8", device)
         out.append(d)
     return out
 
