@@ -480,9 +480,20 @@ __global__ void __launch_bounds__(WC_THREADS) k_win_cut(Prod* __restrict__ prods
     int64_t spw = max((int64_t)1, (tot + P.win.nw - 1) / max((int64_t)1, P.win.nw));
     int64_t nk = max((int64_t)1, (tot + spw - 1) / spw);
     const float binw = (float)(int64_t(1) << P.win.bin_shift);
-    // a CTA's share, and a quarter more: the 6188 x 6188 weighted product (34 of 9539
-    // windows in a bin, a share of 31) is cut well by its bins
-    const bool crowded = (int64_t)s_top > spw * max(WC_CROWD, 5 * nk / (4 * ctas));   // uniform
+    // more than a CTA's share (and a quarter: the 6188 x 6188 weighted product, 34 of 9539
+    // windows in a bin at a share of 31, is cut well by its bins) in windows wider than a
+    // table, or many times that in narrow ones, which are addressed directly and never
+    // halved (a bin of the sums of two simplexes: the sample alone would cost a call of
+    // 0.5 ms 30 us)
+    const int64_t few = spw * max(WC_CROWD, 5 * nk / (4 * ctas)), many = spw * max(WC_DIRECT, 16 * nk / ctas);
+    bool crowded = false;
+    if ((int64_t)s_top > few) {   // uniform
+      for (int i = a; i < b; ++i) {
+        const int64_t x = (int64_t)(hs[i + (i >> 5)] - (i ? hs[(i - 1) + ((i - 1) >> 5)] : 0u));
+        crowded |= x > many || (x > few && x / spw < (int64_t(1) << P.win.bin_shift) / slots);
+      }
+      crowded = __syncthreads_or(crowded);
+    }
     const uint64_t* const ks = (const uint64_t*)hs;
     int64_t nv = 0;   // sampled keys
     if (crowded) {
