@@ -127,7 +127,7 @@ class Clocks:
 # DRAM bytes (read + write) per launch of k_dense_accum on this workload, from
 # one ncu capture of the kernel on it; valid only for the kernel source it was
 # taken on, identified by the leading hex digits of its SHA-256.
-DENSE_TRAFFIC = {"source": "kr_dense.cu", "source_sha256": "9d91294c0d87e967", "bytes": 2740480}
+DENSE_TRAFFIC = {"source": "kr_dense.cu", "source_sha256": "298d521c4405ad08", "bytes": 2838528}
 
 
 def kernel_traffic(rec):
@@ -413,47 +413,15 @@ def main():
         if sel("hash_cfg3"):
             h3 = time_poly(kron, ctx, *workload_cfg3(), dev, stream, flush, "hash_insert",
                            max(3, args.steps // 2))
-            # the windows accumulate on chip and write 16 B per output term
-            roof3 = hbm_roofline("k_window", h3["term_products"], h3["kernel_ms"],
-                                 16.0 * h3["output_terms"] / h3["term_products"], hbm)
-            # the ceiling of a table in device memory on random keys, at this product's
-            # table size (2^24 slots) and key count, and of plain random adds
-            ins = kron.kr_probe_table_update_rate(24, h3["output_terms"], h3["term_products"], 0, local, 3)
-            add = kron.kr_probe_table_update_rate(24, h3["output_terms"], h3["term_products"], 1, local, 3)
-            roof3["ceiling_insert_per_s"] = ins
-            roof3["ceiling_random_add_per_s"] = add
-            # the same random insert-or-adds into a table L2 holds (2^22 slots, 64 MB)
-            roof3["ceiling_insert_l2_table_per_s"] = kron.kr_probe_table_update_rate(
-                22, 1 << 21, h3["term_products"], 0, local, 3)
-            roof3["frac_of_insert_ceiling"] = (h3["term_products"] / (h3["kernel_ms"] * 1e-3)) / ins \
-                if ins > 0 else None
-            h3["roofline"] = roof3
+            h3["roofline"] = window_roofline(h3, hbm)
             paths["hash_cfg3"] = h3
         if sel("poisson_cfg4") or sel("poisson_cfg4_hash") or sel("poisson_cfg4_truncated"):
             f4, g4 = workload_cfg4()
             if sel("poisson_cfg4"):
-                p4 = time_pseries(kron, ctx, f4, g4, dev, stream, flush, 3, hbm_gbs=hbm)
-                # second denominator: random float64 adds into a key-indexed array of
-                # 2^32 8-byte slots (34 GB; the product's array is 46.6 GB), two per pair
-                upd = 2 * p4["term_products"]
-                ceil = kron.kr_probe_table_update_rate(32, min(p4["output_terms"], (7 << 32) // 10), upd, 2,
-                                                       local, 3)
-                p4["roofline"]["ceiling_random_f64_add_per_s"] = ceil
-                p4["roofline"]["frac_of_update_ceiling"] = (upd / (p4["kernel_ms"] * 1e-3)) / ceil \
-                    if ceil > 0 else None
-                paths["poisson_cfg4"] = p4
+                paths["poisson_cfg4"] = time_pseries(kron, ctx, f4, g4, dev, stream, flush, 3, hbm_gbs=hbm)
             if sel("poisson_cfg4_hash"):
-                p4h = time_pseries(kron, ctx, f4, g4, dev, stream, flush, 3, path=kron.KR_PATH_HASH,
-                                   hbm_gbs=hbm)
-                # second denominator: random insert-or-adds (the insert routine, as the
-                # polynomial kernel issues them) into 2^30 16-byte slots, two per pair
-                upd = 2 * p4h["term_products"]
-                ceil = kron.kr_probe_table_update_rate(30, min(p4h["output_terms"], (7 << 30) // 10), upd, 0,
-                                                       local, 3)
-                p4h["roofline"]["ceiling_insert_per_s"] = ceil
-                p4h["roofline"]["frac_of_insert_ceiling"] = (upd / (p4h["kernel_ms"] * 1e-3)) / ceil \
-                    if ceil > 0 else None
-                paths["poisson_cfg4_hash"] = p4h
+                paths["poisson_cfg4_hash"] = time_pseries(kron, ctx, f4, g4, dev, stream, flush, 3,
+                                                          path=kron.KR_PATH_HASH, hbm_gbs=hbm)
             if sel("poisson_cfg4_truncated"):
                 # Sec. 3's truncation of a Poisson product: pairs with |C_f C_g| >= 1e-38 (about 14%
                 # of them; the magnitudes fall with the exponents and multipliers) and terms of
@@ -825,6 +793,16 @@ def hbm_roofline(kernel, units, kms, bytes_per_unit, hbm_gbs, traffic=None):
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy, read + write)"}
 
 
+def window_roofline(r, hbm_gbs):
+    """k_window accumulates on chip and writes 16 B per output term.  Instruction issue bounds it (62% of the issue
+    slots under ncu on the 5000 x 5000-term Poisson product), so its share of the copy rate says only how far HBM is
+    from bounding it."""
+    roof = hbm_roofline("k_window", r["term_products"], r["kernel_ms"], 16.0 * r["output_terms"] / r["term_products"],
+                        hbm_gbs)
+    roof["bound"] = "issue"
+    return roof
+
+
 def time_pseries(kron, ctx, f, g, dev, stream, flush, steps, path=0, hbm_gbs=None, kernel_name=None,
                  **opts):
     import torch
@@ -852,8 +830,8 @@ def time_pseries(kron, ctx, f, g, dev, stream, flush, steps, path=0, hbm_gbs=Non
          "kernel_rate": tp / (kms * 1e-3) / 1e6, "accumulator": form,
          "stages_ms_last_step": dict(ctx.stages())}
     if hbm_gbs:
-        r["roofline"] = hbm_roofline(kernel_name or "k_window", tp, kms,
-                                     16.0 * int(out[3].shape[0]) / tp if windowed else POISSON_BYTES[form], hbm_gbs)
+        r["roofline"] = window_roofline(r, hbm_gbs) if windowed else \
+            hbm_roofline(kernel_name, tp, kms, POISSON_BYTES[form], hbm_gbs)
     return r
 
 

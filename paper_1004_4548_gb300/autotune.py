@@ -1,5 +1,5 @@
 """Autotuner for the per-product knobs: dense or hash path, dense block size,
-hash load factor.
+load factor of a hash table in device memory.
 
 The paper picks the algorithm from the densities of the factors (Sec. 3.2)
 without a threshold; here the choice is measured.  Products are grouped into

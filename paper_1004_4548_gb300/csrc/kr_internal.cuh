@@ -145,7 +145,6 @@ struct Win {
   int32_t kind;          // 0: not windowed
   int32_t swap;          // 1: g is walked and f searched (the shorter factor is walked)
   int32_t merge;         // a CTA may take several windows at once
-  int32_t sparse;        // (not merging) most pairs have a key of their own
   int32_t stage;         // windows of a staged run (0: none)
   int32_t bin_shift;     // histogram bins of 2^bin_shift keys
   int64_t nbins, nw, samples, cap, idx_cap, pt;   // pt: pairs per window
@@ -163,7 +162,8 @@ struct Win {
 };
 
 // A divisor with its reciprocals: floor(2^32 / d) (at most 2^32 - 1) and
-// floor((2^64 - 1) / d).
+// floor((2^64 - 1) / d) (division by an invariant through a high multiply and a
+// correction: Granlund and Montgomery 1994).
 struct Divisor {
   int64_t d;
   uint64_t r64;

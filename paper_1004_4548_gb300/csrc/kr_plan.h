@@ -33,10 +33,17 @@ constexpr double DEFAULT_LOAD = 0.5;
 constexpr int DEFAULT_PROBES = 512;
 // windowed accumulation: terms of the searched factor, and of the walked one
 // (walked once per window, so its length against a window's pairs bounds the
-// searches that find nothing)
+// searches that find nothing).  The crossover with the table in device memory lies
+// beyond both limits: 64 x 2^20 terms take 4.7 against 11.7 ms, 64 x 2^23 40 against
+// 94; 53130 x 53130 weighted terms 42 against 166, 80730 x 80730 104 against 390.
+// Larger products stay with the table, whose memory is bounded by their terms.
 constexpr int64_t WIN_MAX_LIST = int64_t(1) << 20;
 constexpr double WIN_MAX_WALK = 65536.0;
-constexpr int64_t WIN_MIN_ARRAY = int64_t(1) << 24;   // keys of an array of L2's size (128 MB)
+// keys of an array of L2's size (128 MB), for Poisson products: windows and array
+// take 0.65 and 0.50 ms for 3000 x 2200 terms over 1.04e7 keys, 2.04 and 1.27 for
+// 8000 x 7000; over 1.8e8 keys 0.42 and 1.26 (59 keys an update), 0.91 and 1.55 (13),
+// 4.55 and 4.77 (1.6)
+constexpr int64_t WIN_MIN_ARRAY = int64_t(1) << 24;
 constexpr int64_t WIN_MAX_BINS = 32768;   // histogram bins (132 KB of shared memory in the cuts)
 // output room reserved from the bound on the terms up to this many bytes; above
 // it the distinct keys are estimated first

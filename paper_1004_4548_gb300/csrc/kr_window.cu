@@ -11,13 +11,13 @@
 // stretches together in key order: the decode of a single product, or a copy.
 //
 // Measured on GB300 (whole calls): 6188 x 6188 terms of the weighted sparse
-// structure 1.90 -> 1.12 ms, 2311 x 1507 random float64 terms over 2.8e11 keys
-// 12.7 -> 0.45 ms (its ordering alone took 11.9), a Poisson product of 5003 x
-// 3989 terms (37 M output terms) 6.6 -> 2.06 ms, 20000 x 20000 (597 M terms) 64.5
-// -> 45 ms.  The window kernel is bound by instruction issue (60% of the issue
+// structure 1.90 -> 1.05 ms, 2311 x 1507 random float64 terms over 2.8e11 keys
+// 12.7 -> 0.42 ms (its ordering alone took 11.9), a Poisson product of 5003 x
+// 3989 terms (37 M output terms) 6.5 -> 2.0 ms, 20000 x 20000 (597 M terms) 64.5
+// -> 43.5 ms.  The window kernel is bound by instruction issue (62% of the issue
 // slots; 2 CTAs of 512 threads per SM, 110 KB of shared memory each): forming,
-// adding and ordering a pair takes about 20 warp instructions, and the walk over
-// the terms that have no partner in a window adds to it.
+// adding and ordering a pair takes about 20 warp instructions (640 for a row of
+// 32), and the walk over the terms that have no partner in a window adds to it.
 //
 // Pairs of a window.  One factor (the shorter, "A") is walked, the other ("B")
 // is searched: for a term a of A the partners that land in [lo, hi) are the
@@ -1448,7 +1448,7 @@ struct WinRun {
     const WinDesc& D = *P.win.desc;
     const int64_t* start = P.win.start + wfirst;
     const bool narrow = sizeof(KT) == 8 || start[m] - start[0] <= (int64_t)0xfffffff0ll;   // offsets fit
-    const bool sparse = narrow && (P.win.merge ? win_distinct(D, wfirst, D.nw) > 0.5f : P.win.sparse != 0);
+    const bool sparse = narrow && P.win.merge && win_distinct(D, wfirst, D.nw) > 0.5f;
     // (the staging area holds Win::stage windows, at most WST; a run that starts where keys
     // are distinct may go on into a region where they are not, whose windows are
     // weighed otherwise)
