@@ -132,7 +132,10 @@ typedef struct {
   /* The hash path accumulates by windows of the output keys, on chip; setting
    * probe_limit, max_regrow or table_slots asks for one table in device memory
    * (as truncation by coefficients or harmonic order does), which load_factor
-   * and unsorted also concern. */
+   * and unsorted also concern.  The table also takes a product that windows
+   * cannot hold: its pairs fall on too few of its keys, its windows would be cut
+   * into too many pieces, or their room (up to 32 bytes a pair) does not fit in
+   * device memory. */
   double load_factor;    /* hash path: target table load factor, (0, 0.9] */
   int32_t probe_limit;   /* hash path: windows probed before TABLE_FULL */
   int32_t unsorted;      /* hash path: 1 = leave the output in table order */
