@@ -58,6 +58,25 @@ def test_prepared_batch_of_windows_alone(kron, case):
     pb.close()
 
 
+@pytest.mark.parametrize("case", ["swapped", "offsets_64", "dense"])
+def test_replay_keeps_the_statuses_it_finds(kron, case):
+    """Exponents changed in place to a repeated term: the replay reports it, and the next one, mended, does not."""
+    import torch
+    f, g = POLY[case]() if case != "dense" else (random_poly(2, 50, 0, 12, 31), random_poly(2, 60, 0, 12, 32))
+    F, G = up(f), up(g)
+    pb = kron.PreparedBatch([(F, G)])
+    whole = F.exps.clone()
+    for exps, status in ((whole, 0), (torch.cat([whole[:, 1:2], whole[:, 1:]], 1), kron.KR_ERR_DUP), (whole, 0)):
+        F.exps.copy_(exps)
+        pb.launch()
+        torch.cuda.synchronize()
+        r = pb.results()[0]
+        assert r["status"] == status
+        if status == 0:
+            assert_poly_equal(r["exps"], r["coef"], oracle.poly_mul(f, g), case)
+    pb.close()
+
+
 def test_short_estimate_is_repeated(kron, limited):
     """The room comes from an estimate that is always short: every product is repeated with full room."""
     limited(kron.KR_LIMIT_WINDOW_BYTES, 1.0)
