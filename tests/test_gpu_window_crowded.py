@@ -57,6 +57,8 @@ POLY = {
     "offsets_32": lambda: (far(dense_total_degree(4, 8, -100, 100, 1), 1 << 11), far(dense_total_degree(4, 7, -100, 100, 2), 1 << 10)),
     "offsets_64": lambda: (far(dense_total_degree(4, 8, -100, 100, 3), 10 ** 9), far(dense_total_degree(4, 7, -100, 100, 4), 10 ** 9)),
     "both_ends": lambda: (far(dense_total_degree(3, 12, -100, 100, 5), -10 ** 8, 10 ** 8), far(dense_total_degree(3, 11, -100, 100, 6), 10 ** 7)),
+    # 32-bit offsets and a gap of more than 2^32 keys
+    "wide_gap": lambda: (far(dense_total_degree(4, 10, -100, 100, 13), 500000), far(dense_total_degree(4, 10, -100, 100, 14), 480000)),
     "distinct": lambda: (far(random_poly(4, 600, -30, 30, 7), 10 ** 7), far(random_poly(4, 500, -30, 30, 8), -10 ** 7)),
     "a_line": lambda: (far(line(3000, 9), 10 ** 9), far(line(2990, 10), 10 ** 9)),              # 6000 keys: the table
     "wide_line": lambda: (far(line(400, 11), 10 ** 9), far(line(390, 12), 10 ** 9)),            # too few pairs for the table
